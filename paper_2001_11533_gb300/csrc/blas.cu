@@ -260,10 +260,10 @@ template <typename T, typename Z, int TPR>
 __global__ void k_cg2_spmv(MatView<T> A, const Z *__restrict__ z, const T *__restrict__ r, T *__restrict__ s,
                            CgScal *sc, double *partials, unsigned *ticket)
 {
-    pdl_enter();
-    SKIP_DONE();
     int row = my_row<TPR>();
-    T v = row_sum<T, TPR>(A, row, [&](int c) { return (T)__ldg(&z[c]); });
+    RowPre<T> pre;
+    PDL_ENTER_LOADING(&sc->done, (row_prefetch<T, TPR>(A, row, pre)))
+    T v = row_sum_pre<T, TPR>(A, row, pre, [&](int c) { return (T)__ldg(&z[c]); });
     double a[2] = {0.0, 0.0}, tot[2];
     if (row < A.rows && row_leader<TPR>()) {
         s[row] = v;
@@ -281,10 +281,10 @@ __global__ void k_cg2_spmv_df(MatView<float> A, const float *__restrict__ lo, co
                               const double *__restrict__ r, double *__restrict__ s, CgScal *sc, double *partials,
                               unsigned *ticket)
 {
-    pdl_enter();
-    SKIP_DONE();
     int row = my_row<TPR>();
-    double v = row_sum_df<Z, TPR>(A, lo, row, z);
+    RowPreDf pre;
+    PDL_ENTER_LOADING(&sc->done, row_prefetch_df<TPR>(A, lo, row, pre))
+    double v = row_sum_df<Z, TPR>(A, lo, row, pre, z);
     double a[2] = {0.0, 0.0}, tot[2];
     if (row < A.rows && row_leader<TPR>()) {
         s[row] = v;
@@ -721,14 +721,22 @@ __global__ void k_df_start(int n, const double *__restrict__ f, float *__restric
     if (reduce_df_last_block<1>(tot_df, partials, ticket, tot)) cg_finalize(F_START, tot, sc, nullptr);
 }
 
-// K1: s = A z (FP32 z), reduce (r, z) and (z, s) -> alpha, beta
-template <int TPR>
+// K1: s = A z (FP32 z), reduce (r, z) and (z, s) -> alpha, beta.  PRE: the
+// grid covers the rows at once and is one wave, so the row is loaded before
+// the wait for the kernel before (PDL_ENTER_LOADING); the walking form keeps
+// the fewer registers (48 against 64) that its occupancy needs.
+template <int TPR, bool PRE>
 __global__ void k_df_spmv(MatView<float> A, const float *__restrict__ lo, const float *__restrict__ z,
                           const float *__restrict__ rh, const float *__restrict__ rl, float *__restrict__ sh,
                           float *__restrict__ sl, CgScal *sc, double *partials, unsigned *ticket)
 {
-    pdl_enter();
-    SKIP_DONE();
+    RowPreDf pre;
+    if (PRE) {
+        PDL_ENTER_LOADING(&sc->done, row_prefetch_df<TPR>(A, lo, my_row<TPR>(), pre))
+    } else {
+        pdl_enter();
+        SKIP_DONE();
+    }
     // a grid that fits on the GPU at once walks the rows, so each block pays
     // its reduction tail once for several rows per thread
     DF a[2] = {{0.f, 0.f}, {0.f, 0.f}};
@@ -736,6 +744,7 @@ __global__ void k_df_spmv(MatView<float> A, const float *__restrict__ lo, const 
     const int stride = gridDim.x * blockDim.x, slots = A.rows * TPR;
     for (int base = blockIdx.x * blockDim.x; base < slots; base += stride) {
         int row = (base + (int)threadIdx.x) / TPR;
+        if (!PRE) row_prefetch_df<TPR>(A, lo, row, pre);
         bool lead = row < A.rows && row_leader<TPR>();
         float zr = 0.f, rhr = 0.f, rlr = 0.f;
         if (lead) {
@@ -743,13 +752,14 @@ __global__ void k_df_spmv(MatView<float> A, const float *__restrict__ lo, const 
             rhr = rh[row];
             rlr = rl[row];
         }
-        DF v = row_sum_dfv<float, TPR>(A, lo, row, z);
+        DF v = row_sum_dfv<float, TPR>(A, lo, row, pre, z);
         if (lead) {
             sh[row] = v.hi;
             sl[row] = v.lo;
             a[0] = df_add_fast(a[0], df_mulf(DF{rhr, rlr}, zr));
             a[1] = df_add_fast(a[1], df_mulf(v, zr));
         }
+        if (PRE) break;
     }
     if (reduce_df_last_block<2>(a, partials, ticket, tot)) cg_finalize(F_CG2, tot, sc, nullptr);
 }
@@ -871,9 +881,17 @@ int dfcg_spmv(amgh_problem *p, RedSlot &red, const DevCsr &a, const float *z, co
     const int cls = fine_cls(p, n, KC_CGSPMV0, KC_CGSPMV);
     timer_begin(p, cls);
 #define DFSPMV(TPR)                                                                                            \
-    pdl_launch(k_df_spmv<TPR>,                                                                                 \
-               dim3(std::min(rows_grid(n, TPR), resident_grid((const void *)k_df_spmv<TPR>, TPB))), dim3(TPB), \
-               0, p->stream, A, lo, z, hi_of(r), lo_of(r, n), hi_of(s), lo_of(s, n), sc, red.partials, red.ticket)
+    do {                                                                                                       \
+        const int g_ = rows_grid(n, TPR);                                                                      \
+        if (g_ <= PDL_PRELOAD_BLOCKS)                                                                          \
+            pdl_launch(k_df_spmv<TPR, true>, dim3(g_), dim3(TPB), 0, p->stream, A, lo, z, hi_of(r),            \
+                       lo_of(r, n), hi_of(s), lo_of(s, n), sc, red.partials, red.ticket);                      \
+        else                                                                                                   \
+            pdl_launch(k_df_spmv<TPR, false>,                                                                  \
+                       dim3(std::min(g_, resident_grid((const void *)k_df_spmv<TPR, false>, TPB))), dim3(TPB), \
+                       0, p->stream, A, lo, z, hi_of(r), lo_of(r, n), hi_of(s), lo_of(s, n), sc,               \
+                       red.partials, red.ticket);                                                              \
+    } while (0)
     switch (A.tpr) {
     case 2: DFSPMV(2); break;
     case 4: DFSPMV(4); break;

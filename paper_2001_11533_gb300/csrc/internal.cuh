@@ -44,16 +44,39 @@ void amgh_set_capturing(int on);
 // pdl_launch, which lets a kernel be scheduled while its predecessor in the
 // stream (or CUDA graph) is still running; every such kernel calls
 // pdl_enter() first, which waits until the predecessor has completed and its
-// writes are visible, and -- for grids that fit comfortably in one wave --
-// lets its own successor be scheduled right away, so launch latency overlaps
-// the kernel instead of following it.  Without the launch attribute the wait
+// writes are visible, and lets its own successor be scheduled right away, so
+// launch latency overlaps the kernel instead of following it.  (The successor
+// is scheduled once every block of this grid has started, so it takes no
+// place from them; grids above 608 blocks used to hold it back, which cost
+// 0.5 % of the 1025^2 L-shape's step.)  Without the launch attribute the wait
 // returns at once.
-#define PDL_EARLY_BLOCKS 608
 __device__ __forceinline__ void pdl_enter()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (gridDim.x * gridDim.y * gridDim.z <= PDL_EARLY_BLOCKS) asm volatile("griddepcontrol.launch_dependents;" :::);
+    asm volatile("griddepcontrol.launch_dependents;" :::);
 }
+
+// pdl_enter() for a kernel that returns when *flag is set and whose operands
+// that only the setup writes are loaded by `load`.  In a grid of at most
+// PDL_PRELOAD_BLOCKS blocks (four of 256 threads on each of the 152 SMs: one
+// wave) the loads go out before the wait, so they overlap the tail of the
+// kernel before; the flag as it reads before the wait is a hint only: when it
+// is set (an iteration replayed past convergence) nothing is loaded early, and
+// the flag after the wait decides.  Later waves have no wait to overlap and
+// would only be delayed by reading the hint (257^2 FP64 Hessian apply: 5.35 ms
+// with the loads after the wait, 4.65 ms before it; on the 129^3 cube, whose
+// grids have 12 waves, reading the hint in all of them took 22.6 to 24.5 ms).
+#define PDL_PRELOAD_BLOCKS 608
+#define PDL_ENTER_LOADING(flag, load)                                                              \
+    const bool early_ = gridDim.x <= PDL_PRELOAD_BLOCKS && !((flag) && __ldcg((const int *)(flag))); \
+    if (early_) {                                                                                  \
+        load;                                                                                      \
+    }                                                                                              \
+    pdl_enter();                                                                                   \
+    if ((flag) && *(flag)) return;                                                                 \
+    if (!early_) {                                                                                 \
+        load;                                                                                      \
+    }
 
 template <typename... KArgs, typename... Args>
 inline void pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

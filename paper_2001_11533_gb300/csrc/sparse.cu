@@ -434,10 +434,10 @@ int build_lo_parts(Arena &ar, DevCsr &a, cudaStream_t s)
 template <typename T, int TPR>
 __global__ void k_spmv(MatView<T> A, const T *__restrict__ x, T *__restrict__ y, const int *__restrict__ skip)
 {
-    pdl_enter();
-    SKIP_RETURN();
     int r = my_row<TPR>();
-    T v = row_sum<T, TPR>(A, r, [&](int c) { return __ldg(&x[c]); });
+    RowPre<T> pre;
+    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pre)))
+    T v = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return __ldg(&x[c]); });
     if (r < A.rows && row_leader<TPR>()) y[r] = v;
 }
 
@@ -461,19 +461,19 @@ __global__ void k_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *_
                             const T *__restrict__ x, T *__restrict__ d, T *__restrict__ xn, T cdv, T crv,
                             const int *__restrict__ skip)
 {
-    pdl_enter();
-    SKIP_RETURN();
     int r = my_row<TPR>();
     bool lead = r < A.rows && row_leader<TPR>();
-    // row-local operands first, so their loads overlap the row's
-    T br = 0, ir = 0, dr = 0, xr = 0;
+    RowPre<T> pre;
+    T ir = 0;
+    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pre)); ir = lead ? invd[r] : (T)0)
+    // row-local operands first, so their loads overlap the row's gathers
+    T br = 0, dr = 0, xr = 0;
     if (lead) {
         br = b[r];
-        ir = invd[r];
         dr = d[r];
         xr = x[r];
     }
-    T ax = row_sum<T, TPR>(A, r, [&](int c) { return __ldg(&x[c]); });
+    T ax = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return __ldg(&x[c]); });
     if (lead) {
         T dn, xv;
         cheb_point(br, ax, ir, dr, xr, cdv, crv, dn, xv);
@@ -524,8 +524,6 @@ __global__ void __launch_bounds__(32 * ELL_SLICES)
                     const float *__restrict__ invd, const float *__restrict__ b, const float *__restrict__ x,
                     float *__restrict__ d, float *__restrict__ xn, float cdv, float crv, const int *__restrict__ skip)
 {
-    pdl_enter();
-    if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char ell_sm[];
     __shared__ __align__(8) uint64_t bar;
     const int first_polls = *(volatile int *)&g_bulk_first_polls; // issued early: off the wait's path
@@ -536,18 +534,29 @@ __global__ void __launch_bounds__(32 * ELL_SLICES)
     float *sv = (float *)ell_sm;
     unsigned char *sc = ell_sm + (size_t)ELL_SLICES * 32 * W * sizeof(float);
     const uint32_t ib = D16 ? 2 : 4;
-    if (threadIdx.x == 0) {
+    const int row = s0 * 32 + (int)threadIdx.x;
+    const bool ok = row < rows;
+    // the matrix and D^-1 are the setup's: their copies and loads go out before
+    // the wait for the kernel before (unless the iteration is one replayed past
+    // convergence, as PDL_ENTER_LOADING), and only the vectors come after it
+    auto stage = [&]() {
         mbar_init(&bar, 1);
         mbar_expect_tx(&bar, nent * (4 + ib));
         bulk_g2s(sv, v + first, nent * 4, &bar);
         bulk_g2s(sc, (const unsigned char *)cols + first * ib, nent * ib, &bar);
+    };
+    const bool early = threadIdx.x == 0 && !(skip && __ldcg(skip));
+    if (early) stage();
+    const float ir = ok ? invd[row] : 0.f;
+    pdl_enter();
+    if (skip && *skip) {
+        if (early) mbar_wait(&bar, 0, BULK_DRAIN_POLLS); // no copy may outlive its block
+        return;
     }
-    const int row = s0 * 32 + (int)threadIdx.x;
-    const bool ok = row < rows;
-    float br = 0.f, ir = 0.f, dr = 0.f, xr = 0.f;
+    if (threadIdx.x == 0 && !early) stage();
+    float br = 0.f, dr = 0.f, xr = 0.f;
     if (ok) {
         br = b[row];
-        ir = invd[row];
         dr = d[row];
         xr = x[row];
     }
@@ -582,12 +591,12 @@ template <typename T, int TPR>
 __global__ void k_residual(MatView<T> A, const T *__restrict__ b, const T *__restrict__ x, T *__restrict__ res,
                            const int *__restrict__ skip)
 {
-    pdl_enter();
-    SKIP_RETURN();
     int r = my_row<TPR>();
     bool lead = r < A.rows && row_leader<TPR>();
+    RowPre<T> pre;
+    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pre)))
     T br = lead ? b[r] : (T)0;
-    T ax = row_sum<T, TPR>(A, r, [&](int c) { return __ldg(&x[c]); });
+    T ax = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return __ldg(&x[c]); });
     if (lead) res[r] = rsub(br, ax);
 }
 
@@ -598,12 +607,12 @@ __global__ void k_restrict_first(MatView<T> St, const T *__restrict__ r, T *__re
                                  const T *__restrict__ invd, T *__restrict__ d, T *__restrict__ x, T c0,
                                  const int *__restrict__ skip)
 {
-    pdl_enter();
-    SKIP_RETURN();
     int i = my_row<TPR>();
     bool lead = i < St.rows && row_leader<TPR>();
-    T ir = lead ? invd[i] : (T)0;
-    T b = row_sum<T, TPR>(St, i, [&](int c) { return __ldg(&r[c]); });
+    RowPre<T> pre;
+    T ir = 0;
+    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(St, i, pre)); ir = lead ? invd[i] : (T)0)
+    T b = row_sum_pre<T, TPR>(St, i, pre, [&](int c) { return __ldg(&r[c]); });
     if (lead) {
         bc[i] = b;
         T v = cheb_first_point(b, ir, c0);
@@ -616,12 +625,12 @@ template <typename T, int TPR>
 __global__ void k_prolong_add(MatView<T> S, const T *__restrict__ e, T *__restrict__ x,
                               const int *__restrict__ skip)
 {
-    pdl_enter();
-    SKIP_RETURN();
     int i = my_row<TPR>();
     bool lead = i < S.rows && row_leader<TPR>();
+    RowPre<T> pre;
+    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(S, i, pre)))
     T xi = lead ? x[i] : (T)0;
-    T v = row_sum<T, TPR>(S, i, [&](int c) { return __ldg(&e[c]); });
+    T v = row_sum_pre<T, TPR>(S, i, pre, [&](int c) { return __ldg(&e[c]); });
     if (lead) x[i] = radd(xi, v);
 }
 
@@ -647,11 +656,11 @@ template <bool VEC>
 __global__ void k_dense_gemv32(int n, int ld, const float *__restrict__ inv, const float *__restrict__ b,
                                float *__restrict__ x, const int *__restrict__ skip)
 {
-    pdl_enter();
-    SKIP_RETURN();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    DensePre pre;
+    PDL_ENTER_LOADING(skip, if (warp < n) dense_prefetch(inv, ld, warp, n, lane, pre))
     if (warp >= n) return;
-    float acc = dense_row32<VEC>(inv, ld, warp, n, b, lane);
+    float acc = dense_row32<VEC>(inv, ld, warp, n, b, lane, pre);
     if (lane == 0) x[warp] = acc;
 }
 

@@ -85,41 +85,79 @@ __device__ __forceinline__ bool row_leader()
     return TPR == 1 || (threadIdx.x & (TPR - 1)) == 0;
 }
 
-// sum_j a_rj * xf(j); every lane of the group returns the row's value.  All
-// lanes of a warp must call this (rows past the end contribute zero).
+// The first chunk of a lane's row: entry range, values and columns.  A matrix
+// is written by the setup only, which ends with a stream synchronisation, so a
+// solve-phase kernel may load it before pdl_enter(): the loads of a row's
+// pointers, values and columns (three dependent trips to memory) then overlap
+// the tail of the kernel before, and only the gathers of the vector remain
+// after the wait.
+template <typename T>
+struct RowPre {
+    int k, end;
+    T vv[ROW_UNROLL];
+    int cc[ROW_UNROLL];
+};
+
+template <typename T, int TPR>
+__device__ __forceinline__ void row_load(const MatView<T> &m, int row, int k0, int end, RowPre<T> &p)
+{
+    constexpr int STEP = TPR == 1 ? 32 : TPR;
+#pragma unroll
+    for (int j = 0; j < ROW_UNROLL; j++) {
+        bool ok = k0 + STEP * j < end;
+        p.vv[j] = ok ? m.v[k0 + STEP * j] : (T)0;
+        p.cc[j] = ok ? col_of(m, row, k0 + STEP * j) : 0;
+    }
+}
+
+template <typename T, int TPR>
+__device__ __forceinline__ void row_prefetch(const MatView<T> &m, int row, RowPre<T> &p)
+{
+    p.k = p.end = 0;
+    if (row < m.rows) {
+        lane_range<T, TPR>(m, row, p.k, p.end);
+        row_load<T, TPR>(m, row, p.k, p.end, p);
+    }
+}
+
+// sum_j a_rj * xf(j) from a prefetched row; every lane of the group returns
+// the row's value.  All lanes of a warp must call this (rows past the end
+// contribute zero).
 template <typename T, int TPR, typename F>
-__device__ __forceinline__ T row_sum(const MatView<T> &m, int row, F xf)
+__device__ __forceinline__ T row_sum_pre(const MatView<T> &m, int row, RowPre<T> &p, F xf)
 {
     constexpr int STEP = TPR == 1 ? 32 : TPR;
     T acc = (T)0;
     if (row < m.rows) {
-        int k, end;
-        lane_range<T, TPR>(m, row, k, end);
+        const int end = p.end;
         auto chunk = [&](int k0) {
-            T vv[ROW_UNROLL];
-            int cc[ROW_UNROLL];
-#pragma unroll
-            for (int j = 0; j < ROW_UNROLL; j++) {
-                bool ok = k0 + STEP * j < end;
-                vv[j] = ok ? m.v[k0 + STEP * j] : (T)0;
-                cc[j] = ok ? col_of(m, row, k0 + STEP * j) : 0;
-            }
             T xv[ROW_UNROLL];
 #pragma unroll
-            for (int j = 0; j < ROW_UNROLL; j++) xv[j] = k0 + STEP * j < end ? xf(cc[j]) : (T)0;
+            for (int j = 0; j < ROW_UNROLL; j++) xv[j] = k0 + STEP * j < end ? xf(p.cc[j]) : (T)0;
 #pragma unroll
             for (int j = 0; j < ROW_UNROLL; j++)
-                if (k0 + STEP * j < end) acc += vv[j] * xv[j];
+                if (k0 + STEP * j < end) acc += p.vv[j] * xv[j];
         };
-        if (m.wmax <= ROW_UNROLL) chunk(k);
-        else
-            for (; k < end; k += STEP * ROW_UNROLL) chunk(k);
+        chunk(p.k);
+        if (m.wmax > ROW_UNROLL)
+            for (int k = p.k + STEP * ROW_UNROLL; k < end; k += STEP * ROW_UNROLL) {
+                row_load<T, TPR>(m, row, k, end, p);
+                chunk(k);
+            }
     }
     if (TPR > 1) {
 #pragma unroll
         for (int o = TPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, TPR);
     }
     return acc;
+}
+
+template <typename T, int TPR, typename F>
+__device__ __forceinline__ T row_sum(const MatView<T> &m, int row, F xf)
+{
+    RowPre<T> p;
+    row_prefetch<T, TPR>(m, row, p);
+    return row_sum_pre<T, TPR>(m, row, p, xf);
 }
 
 // a z added to acc, a = ahi + alo (FP32 parts of an FP64 value)
@@ -135,37 +173,57 @@ __device__ __forceinline__ void df_term<double>(DF &acc, float ahi, float alo, d
     df_fma2(acc, ahi, alo, zhi, zlo);
 }
 
-// sum_j a_rj z_j in double-float, not normalised; every lane of the group
-// returns it
+// A prefetched row with the low parts of its values (row_prefetch)
+struct RowPreDf {
+    RowPre<float> h;
+    float vl[ROW_UNROLL];
+};
+
+template <int TPR>
+__device__ __forceinline__ void row_load_df(const MatView<float> &m, const float *__restrict__ lo, int row, int k0,
+                                            int end, RowPreDf &p)
+{
+    constexpr int STEP = TPR == 1 ? 32 : TPR;
+    row_load<float, TPR>(m, row, k0, end, p.h);
+#pragma unroll
+    for (int j = 0; j < ROW_UNROLL; j++) p.vl[j] = k0 + STEP * j < end ? lo[k0 + STEP * j] : 0.f;
+}
+
+template <int TPR>
+__device__ __forceinline__ void row_prefetch_df(const MatView<float> &m, const float *__restrict__ lo, int row,
+                                                RowPreDf &p)
+{
+    p.h.k = p.h.end = 0;
+    if (row < m.rows) {
+        lane_range<float, TPR>(m, row, p.h.k, p.h.end);
+        row_load_df<TPR>(m, lo, row, p.h.k, p.h.end, p);
+    }
+}
+
+// sum_j a_rj z_j in double-float from a prefetched row, not normalised; every
+// lane of the group returns it
 template <typename Z, int TPR>
 __device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             const Z *__restrict__ z)
+                                             RowPreDf &p, const Z *__restrict__ z)
 {
     constexpr int STEP = TPR == 1 ? 32 : TPR;
     DF acc = {0.f, 0.f};
     if (row < m.rows) {
-        int k, end;
-        lane_range<float, TPR>(m, row, k, end);
+        const int end = p.h.end;
         auto chunk = [&](int k0) {
-            float vh[ROW_UNROLL], vl[ROW_UNROLL];
-            int cc[ROW_UNROLL];
-#pragma unroll
-            for (int j = 0; j < ROW_UNROLL; j++) {
-                bool ok = k0 + STEP * j < end;
-                vh[j] = ok ? m.v[k0 + STEP * j] : 0.f;
-                vl[j] = ok ? lo[k0 + STEP * j] : 0.f;
-                cc[j] = ok ? col_of(m, row, k0 + STEP * j) : 0;
-            }
             Z zv[ROW_UNROLL];
 #pragma unroll
-            for (int j = 0; j < ROW_UNROLL; j++) zv[j] = k0 + STEP * j < end ? __ldg(&z[cc[j]]) : (Z)0;
+            for (int j = 0; j < ROW_UNROLL; j++) zv[j] = k0 + STEP * j < end ? __ldg(&z[p.h.cc[j]]) : (Z)0;
 #pragma unroll
             for (int j = 0; j < ROW_UNROLL; j++)
-                if (k0 + STEP * j < end) df_term<Z>(acc, vh[j], vl[j], zv[j]);
+                if (k0 + STEP * j < end) df_term<Z>(acc, p.h.vv[j], p.vl[j], zv[j]);
         };
-        if (m.wmax <= ROW_UNROLL) chunk(k);
-        else
-            for (; k < end; k += STEP * ROW_UNROLL) chunk(k);
+        chunk(p.h.k);
+        if (m.wmax > ROW_UNROLL)
+            for (int k = p.h.k + STEP * ROW_UNROLL; k < end; k += STEP * ROW_UNROLL) {
+                row_load_df<TPR>(m, lo, row, k, end, p);
+                chunk(k);
+            }
     }
     if (TPR > 1) {
 #pragma unroll
@@ -180,9 +238,9 @@ __device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const floa
 // sum_j a_rj z_j in double-float (normalised)
 template <typename Z, int TPR>
 __device__ __forceinline__ DF row_sum_dfv(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                          const Z *__restrict__ z)
+                                          RowPreDf &p, const Z *__restrict__ z)
 {
-    DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, z);
+    DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, p, z);
     DF r;
     quick_two_sum(acc.hi, acc.lo, r.hi, r.lo);
     return r;
@@ -190,9 +248,9 @@ __device__ __forceinline__ DF row_sum_dfv(const MatView<float> &m, const float *
 
 template <typename Z, int TPR>
 __device__ __forceinline__ double row_sum_df(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             const Z *__restrict__ z)
+                                             RowPreDf &p, const Z *__restrict__ z)
 {
-    DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, z);
+    DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, p, z);
     return (double)acc.hi + (double)acc.lo;
 }
 
@@ -224,27 +282,57 @@ __device__ __forceinline__ T cheb_first_point(T br, T ir, T c)
 }
 
 // one row of a dense FP32 inverse (rows padded to ld, 16-byte aligned) times
-// b; the whole warp returns the sum
+// b; the whole warp returns the sum.  The row's first DENSE_PRE groups of four
+// per lane (1024 entries in all) are loaded by dense_prefetch, which needs
+// only the setup's data and so may run before pdl_enter().
+#define DENSE_PRE 8
+struct DensePre {
+    float4 r[DENSE_PRE];
+};
+
+__device__ __forceinline__ void dense_prefetch(const float *__restrict__ inv, int ld, int row, int n, int lane,
+                                               DensePre &p)
+{
+    const float4 *r4 = reinterpret_cast<const float4 *>(inv + (int64_t)row * ld);
+    const int full = n >> 2;
+#pragma unroll
+    for (int j = 0; j < DENSE_PRE; j++)
+        if (lane + 32 * j < full) p.r[j] = r4[lane + 32 * j];
+}
+
 template <bool VEC>
 __device__ __forceinline__ float dense_row32(const float *__restrict__ inv, int ld, int row, int n, const float *b,
-                                             int lane)
+                                             int lane, const DensePre &p)
 {
     const float4 *r4 = reinterpret_cast<const float4 *>(inv + (int64_t)row * ld);
     int full = n >> 2;
     float a0 = 0.f, a1 = 0.f;
-    for (int k = lane; k < full; k += 32) {
-        float4 r = r4[k], v;
+    auto term = [&](int k, const float4 &r) {
+        float4 v;
         if (VEC) v = __ldcg(reinterpret_cast<const float4 *>(b) + k);
         else v = make_float4(__ldcg(b + 4 * k), __ldcg(b + 4 * k + 1), __ldcg(b + 4 * k + 2), __ldcg(b + 4 * k + 3));
         a0 = fmaf(r.x, v.x, a0);
         a1 = fmaf(r.y, v.y, a1);
         a0 = fmaf(r.z, v.z, a0);
         a1 = fmaf(r.w, v.w, a1);
-    }
+    };
+#pragma unroll
+    for (int j = 0; j < DENSE_PRE; j++)
+        if (lane + 32 * j < full) term(lane + 32 * j, p.r[j]);
+    for (int k = lane + 32 * DENSE_PRE; k < full; k += 32) term(k, r4[k]);
     for (int k = (full << 2) + lane; k < n; k += 32) a0 = fmaf(inv[(int64_t)row * ld + k], __ldcg(b + k), a0);
     float acc = a0 + a1;
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     return acc;
+}
+
+template <bool VEC>
+__device__ __forceinline__ float dense_row32(const float *__restrict__ inv, int ld, int row, int n, const float *b,
+                                             int lane)
+{
+    DensePre p;
+    dense_prefetch(inv, ld, row, n, lane, p);
+    return dense_row32<VEC>(inv, ld, row, n, b, lane, p);
 }
 
 inline int rows_grid(int rows, int tpr, int tpb = 256) { return ceil_div((int64_t)rows * (tpr < 1 ? 1 : tpr), tpb); }
