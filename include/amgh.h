@@ -132,7 +132,9 @@ typedef struct {
  *                  handles from amgh_problem_share and the batch runtime's
  *                  handles use 0.  Same arithmetic per row, sums grouped
  *                  differently: results agree with 0 to the CG tolerance, not
- *                  to the bit */
+ *                  to the bit.  Single-column mass CGs on levels small enough
+ *                  for one thread-block cluster (up to 16384 lanes of at most
+ *                  16 entries) are one cluster launch with either value */
 typedef struct {
     int max_levels;
     int hessian_levels;

@@ -183,6 +183,7 @@ struct DevCsr {
     // the widest slice; CSR: ceil(longest row / tpr)); rows up to
     // ROW_UNROLL per lane are read with every load issued up front
     int wmax = 1 << 30;
+    int longest = 0; // entries of the longest CSR row (0: not known)
     // SELL-32; ellw > 0: every slice has this width (slice s starts at
     // 32 * ellw * s, so kernels need not load the slice pointers)
     int nslices = 0, sell_nnz = 0, ellw = 0;
@@ -509,6 +510,14 @@ int vec_fill(amgh_problem *p, int n, double v, double *x);
 int vec_dot(amgh_problem *p, RedSlot &red, int n, const double *x, const double *y, double *out_dev);
 int scatter_state(amgh_problem *p, int m, const int *vertex_of_state, const double *ys,
                   double *full, double scale_add_beta_u, const double *u);
+
+// ------------------------------------------------------------------ mass.cu
+// whether the mass CG of this level runs as one cluster launch; the launch:
+// cols right sides interleaved (element i of column c at i * cols + c), the
+// final scalars of column c in sc[c]
+bool mass_cluster_fits(const DevCsr &a, bool df);
+int mass_cluster(amgh_problem *p, const CtrlLevel &C, bool df, const double *b, double *x, CgScal *sc, int cols,
+                 double tol, int maxit);
 
 // ------------------------------------------------------------------ assemble.cu
 int assemble_full(amgh_problem *p);

@@ -520,6 +520,20 @@ int mass_solve(amgh_problem *p, int l, const double *b, double *x, int64_t *iter
     int n = C.Mu.rows;
     // precision 2: the mass CG in double-float too, Jacobi from FP32 copies
     bool df = p->aopts.precision == 2;
+    if (mass_cluster_fits(C.Mu, df)) {
+        timer_begin(p, KC_VEC);
+        TRY(mass_cluster(p, C, df, b, x, C.mscal, 1, p->sopts.mass_tol, p->sopts.mass_max_iter));
+        timer_end(p, KC_VEC, 48.0 * n);
+        CgScal h;
+        TRY(read_scal(p, C.mscal, &h));
+        // per iteration as the graph-replayed pair: the product with its dots, the update
+        const double mat = df ? spmv_bytes(C.Mu, 4) + 4.0 * C.Mu.nnz : spmv_bytes(C.Mu, 8);
+        count_bytes(h.iters * (mat + (df ? 96.0 : 112.0) * n));
+        p->c_mass_lvl[l] += h.iters;
+        p->c_mass += h.iters;
+        if (iters) *iters = h.iters;
+        return cg_status(h);
+    }
     if (df && p->aopts.persistent_cg && !p->parent && !p->in_batch && !p->capturing)
         return persistent_mass_single(p, l, b, x, iters);
     if (df) {

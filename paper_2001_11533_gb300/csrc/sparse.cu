@@ -383,6 +383,7 @@ static int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
     double avg = a.rows > 0 ? (double)a.nnz / a.rows : 0.0;
     int longest = 0;
     TRY(max_row_length(a, s, &longest));
+    a.longest = longest;
     // SELL-32 for short rows, and for rows up to 16 long when every row has
     // nearly the longest length (uniform-width SELL: the staged smoother);
     // otherwise CSR with 4..32 lanes per row

@@ -200,11 +200,11 @@ __device__ __forceinline__ void row_prefetch_df(const MatView<float> &m, const f
     }
 }
 
-// sum_j a_rj z_j in double-float from a prefetched row, not normalised; every
-// lane of the group returns it
-template <typename Z, int TPR>
-__device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             RowPreDf &p, const Z *__restrict__ z)
+// sum_j a_rj xf(j) in double-float from a prefetched row, not normalised;
+// every lane of the group returns it
+template <typename Z, int TPR, typename F>
+__device__ __forceinline__ DF row_sum_df_xf(const MatView<float> &m, const float *__restrict__ lo, int row,
+                                            RowPreDf &p, F xf)
 {
     constexpr int STEP = TPR == 1 ? 32 : TPR;
     DF acc = {0.f, 0.f};
@@ -213,7 +213,7 @@ __device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const floa
         auto chunk = [&](int k0) {
             Z zv[ROW_UNROLL];
 #pragma unroll
-            for (int j = 0; j < ROW_UNROLL; j++) zv[j] = k0 + STEP * j < end ? __ldg(&z[p.h.cc[j]]) : (Z)0;
+            for (int j = 0; j < ROW_UNROLL; j++) zv[j] = k0 + STEP * j < end ? xf(p.h.cc[j]) : (Z)0;
 #pragma unroll
             for (int j = 0; j < ROW_UNROLL; j++)
                 if (k0 + STEP * j < end) df_term<Z>(acc, p.h.vv[j], p.vl[j], zv[j]);
@@ -233,6 +233,13 @@ __device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const floa
         }
     }
     return acc;
+}
+
+template <typename Z, int TPR>
+__device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const float *__restrict__ lo, int row,
+                                             RowPreDf &p, const Z *__restrict__ z)
+{
+    return row_sum_df_xf<Z, TPR>(m, lo, row, p, [&](int c) { return __ldg(&z[c]); });
 }
 
 // sum_j a_rj z_j in double-float (normalised)

@@ -103,3 +103,46 @@ __device__ bool reduce_last_block(const double (&val)[NV], double *partials, uns
     if (threadIdx.x == 0) *ticket = 0u;
     return threadIdx.x == 0;
 }
+
+// Order of non-negative FP64 numbers by their bits: an FP64 comparison, like
+// every FP64 instruction, holds its unit for ~65 cycles here.
+__device__ __forceinline__ bool pos64(double x) // 0 < x <= infinity
+{
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool le64(double x, double y) // x <= y, both >= 0
+{
+    return __double_as_longlong(x) <= __double_as_longlong(y);
+}
+
+// alpha and beta of the single-reduction CG (Chronopoulos & Gear) from
+// g = (r, z), d = (z, A z) and, from the step before (k1 > 0), rz = g' and
+// ra = g' alpha':
+//   beta = g / g',  alpha = g / (d - beta g / alpha') = g ra / (d ra - g^2).
+// Called by all lanes of one warp with the same arguments; all get the result.
+// An FP64 division takes ten dependent FP64 instructions, so the two divisions
+// are made by two lanes of one instruction sequence (in the textbook order
+// three divisions follow each other).  The products are formed on g and ra
+// scaled by the power of two of g, so that no square over- or underflows where
+// g itself does not.  Returns CG_RUNNING, or the status that ends the loop.
+__device__ __forceinline__ int cg2_scalars(double g, double d, int k1, double rz, double ra, double &alpha,
+                                           double &beta)
+{
+    double num = g, den = d;
+    if (k1) {
+        const int e = (__double2hiint(g) >> 20) & 0x7ff; // biased exponent
+        const double s = __hiloint2double(min(max(2046 - e, 1), 2046) << 20, 0);
+        const double gs = g * s, rs = ra * s;
+        num = gs * rs;
+        den = fma(d * s, rs, -(gs * gs));
+    }
+    const bool second = threadIdx.x & 1;
+    const double quo = (second ? g : num) / (second ? rz : den);
+    alpha = __shfl_sync(0xffffffffu, quo, 0);
+    beta = __shfl_sync(0xffffffffu, quo, 1);
+    if (!k1) beta = 0.0;
+    if (pos64(g) && pos64(d) && pos64(den)) return CG_RUNNING;
+    return finite64(g) && finite64(d) && finite64(den) ? CG_INDEFINITE : CG_NUMERIC;
+}
