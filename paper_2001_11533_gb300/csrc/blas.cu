@@ -61,8 +61,37 @@ enum {
 
 __device__ __forceinline__ bool bad(double x) { return !(x == x) || isinf(x); }
 
+// Called by the first warp of the block that finished last; lane 0 acts, but
+// the alpha / beta step uses all lanes (cg2_scalars).
 __device__ void cg_finalize(int mode, const double *t, CgScal *sc, double *out)
 {
+    if (mode == F_CG2) {
+        const double g = t[0];
+        const int k1 = sc->k1;
+        double alpha, beta;
+        const int status = cg2_scalars(g, t[1], k1, sc->rz, sc->ra, alpha, beta);
+        __syncwarp(); // every lane has read the scalars
+        const int l = threadIdx.x & 31;
+        if (status != CG_RUNNING) {
+            if (l == 0) {
+                sc->status = status;
+                sc->done = 1;
+            }
+        } else if (l == 0) {
+            sc->ahi = (float)alpha;
+            sc->alo = (float)(alpha - (double)(float)alpha);
+            sc->rz = g;
+            sc->ra = g * alpha;
+            sc->alpha = alpha;
+            sc->k1 = k1 + 1;
+        } else if (l == 1) {
+            sc->bhi = (float)beta;
+            sc->blo = (float)(beta - (double)(float)beta);
+            sc->beta = beta;
+        }
+        return;
+    }
+    if (threadIdx.x & 31) return;
     switch (mode) {
     case F_START:
     case F_MASS_START: {
@@ -113,10 +142,10 @@ __device__ void cg_finalize(int mode, const double *t, CgScal *sc, double *out)
         sc->rr = t[0];
         sc->iters += 1;
         sc->total_iters += 1;
-        if (bad(t[0])) {
+        if (!finite64(t[0])) {
             sc->status = CG_NUMERIC;
             sc->done = 1;
-        } else if (t[0] <= sc->thr) {
+        } else if (le64(t[0], sc->thr)) { // sums of squares
             sc->status = CG_CONVERGED;
             sc->done = 1;
         } else if (sc->iters >= sc->maxit) {
@@ -183,36 +212,6 @@ __device__ void cg_finalize(int mode, const double *t, CgScal *sc, double *out)
     case F_SCALE: {
         double nrm = sqrt(t[0]);
         sc->scale = (nrm > 0.0 && !bad(nrm)) ? exp2(-rint(log2(nrm))) : 1.0;
-        break;
-    }
-    case F_CG2: {
-        double g = t[0], d = t[1];
-        if (!(g > 0.0) || !(d > 0.0)) {
-            sc->status = (bad(g) || bad(d)) ? CG_NUMERIC : CG_INDEFINITE;
-            sc->done = 1;
-            break;
-        }
-        double beta = 0.0, alpha;
-        if (sc->k1 == 0) {
-            alpha = g / d;
-        } else {
-            beta = g / sc->rz;
-            double den = d - beta * g / sc->alpha;
-            if (!(den > 0.0)) {
-                sc->status = bad(den) ? CG_NUMERIC : CG_INDEFINITE;
-                sc->done = 1;
-                break;
-            }
-            alpha = g / den;
-        }
-        sc->rz = g;
-        sc->alpha = alpha;
-        sc->beta = beta;
-        sc->k1 += 1;
-        sc->ahi = (float)alpha;
-        sc->alo = (float)(alpha - (double)sc->ahi);
-        sc->bhi = (float)beta;
-        sc->blo = (float)(beta - (double)sc->bhi);
         break;
     }
     }
@@ -307,7 +306,7 @@ __global__ void k_cg2_update(int n, Z *__restrict__ z, const T *__restrict__ s, 
     pdl_enter();
     SKIP_DONE();
     T a = (T)sc->alpha, b = (T)sc->beta;
-    bool first = sc->beta == 0.0;
+    const bool first = sc->k1 == 1;
     double v[1] = {0.0}, tot[1];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         T zi = (T)z[i];
@@ -779,7 +778,7 @@ __global__ void k_df_update(int n, const float *z, const float *__restrict__ sh,
     SKIP_DONE();
     DF al = {sc->ahi, sc->alo}, be = {sc->bhi, sc->blo};
     DF nal = {-al.hi, -al.lo};
-    bool first = sc->beta == 0.0;
+    const bool first = sc->k1 == 1;
     DF acc = {0.f, 0.f}, tot_df[1];
     double tot[1];
     // operands of one element: z, s, p, q, x, r (hi/lo) and D^-1

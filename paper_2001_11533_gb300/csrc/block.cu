@@ -339,10 +339,10 @@ __device__ __forceinline__ void row_sum_df_k(const MatView<float> &m, const floa
 // TPB threads).  Inside a block the values go through shared memory and warp
 // w sums values w, w + 8, ... (fewer FP64 adds than NV butterflies); block
 // partials ([NV][gridDim.x]) are summed in fixed order by the last block to
-// finish, which issues all NV loads of a pass together.  Returns true in
-// thread 0 of that block, with the sums in tot.
+// finish, which issues all NV loads of a pass together.  Returns true in the
+// first warp of that block, with the sums in shared memory at tot.
 template <int NV>
-__device__ bool reduce_k(const double (&val)[NV], double *partials, unsigned *ticket, double (&tot)[NV])
+__device__ bool reduce_k(const double (&val)[NV], double *partials, unsigned *ticket, const double *&tot)
 {
     __shared__ double sh[NV][TPB_K];
     __shared__ double stot[NV];
@@ -382,10 +382,9 @@ __device__ bool reduce_k(const double (&val)[NV], double *partials, unsigned *ti
         if (l == 0) stot[q] = u;
     }
     __syncthreads();
-    if (t != 0) return false;
-#pragma unroll
-    for (int q = 0; q < NV; q++) tot[q] = stot[q];
-    *ticket = 0u;
+    if (t >= 32) return false;
+    if (t == 0) *ticket = 0u;
+    tot = stot;
     return true;
 }
 
@@ -398,7 +397,7 @@ __device__ bool reduce_k(const double (&val)[NV], double *partials, unsigned *ti
 template <int NV>
 struct DfStage {
     float hi[NV][TPB_K], lo[NV][TPB_K];
-    DF tot[NV];
+    double tot[NV]; // the sums over all blocks
 };
 
 template <int NV, int NVMAX = NV>
@@ -423,14 +422,13 @@ __device__ void block_df_partials(const DF (&val)[NV], float2 *part, int nb, int
     }
 }
 
-// the NV sums over the nb block partials, in fixed order; thread 0 returns them
+// the NV sums over the nb block partials, in fixed order, to st.tot
 template <int NV, int NVMAX = NV>
-__device__ void sum_df_partials(const float2 *part, int nb, double (&tot)[NV], DfStage<NVMAX> &st)
+__device__ void sum_df_partials(const float2 *part, int nb, DfStage<NVMAX> &st)
 {
     static_assert(NV <= NVMAX, "staging buffer too small");
     float(&shh)[NVMAX][TPB_K] = st.hi;
     float(&shl)[NVMAX][TPB_K] = st.lo;
-    DF(&stot)[NVMAX] = st.tot;
     const int t = threadIdx.x, w = t >> 5, l = t & 31;
     __syncthreads(); // the staging buffer may still be read by a previous step
     DF s[NV];
@@ -454,17 +452,13 @@ __device__ void sum_df_partials(const float2 *part, int nb, double (&tot)[NV], D
 #pragma unroll
         for (int j = l; j < TPB_K; j += 32) u = df_add_fast(u, DF{shh[q][j], shl[q][j]});
         u = df_warp_sum(u);
-        if (l == 0) stot[q] = u;
+        if (l == 0) st.tot[q] = df_to_double(u);
     }
     __syncthreads();
-    if (t == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; q++) tot[q] = df_to_double(stot[q]);
-    }
 }
 
 template <int NV>
-__device__ bool reduce_dfk(const DF (&val)[NV], double *partials, unsigned *ticket, double (&tot)[NV])
+__device__ bool reduce_dfk(const DF (&val)[NV], double *partials, unsigned *ticket, const double *&tot)
 {
     __shared__ bool is_last;
     __shared__ DfStage<NV> st;
@@ -477,127 +471,121 @@ __device__ bool reduce_dfk(const DF (&val)[NV], double *partials, unsigned *tick
     __syncthreads();
     if (!is_last) return false;
     __threadfence();
-    sum_df_partials<NV>(part, nb, tot, st);
-    if (t != 0) return false;
-    *ticket = 0u;
+    sum_df_partials<NV>(part, nb, st);
+    if (t >= 32) return false;
+    if (t == 0) *ticket = 0u;
+    tot = st.tot;
     return true;
 }
 
 // ------------------------------------------------------------------ finalisers
 __device__ __forceinline__ bool nonfinite(double x) { return !(x == x) || isinf(x); }
 
-template <int K>
-__device__ void bs_all(BScal *bs)
+// The finalisers are called by one whole warp, with the sums of all blocks at
+// t: lane c takes the scalar step of column c (lanes 2c and 2c + 1 the alpha /
+// beta step, cg2_scalars).  FP64 scalar code is ~100 cycles an instruction
+// here: looping over eight columns in one thread took 16 us of an iteration.
+__device__ __forceinline__ void bs_all(BScal *bs, int done)
 {
-    int a = 1;
-#pragma unroll
-    for (int c = 0; c < K; c++) a &= bs->c[c].done != 0;
-    bs->all = a;
+    const int all = __all_sync(0xffffffffu, done);
+    if ((threadIdx.x & 31) == 0) bs->all = all;
 }
 
 // f.f per column: stopping threshold tol^2 f.f; a zero column has converged
 // df: the CG runs on the right side scaled by `scale` (double-float vectors),
 // so r.r and the threshold are kept in scaled units
 template <int K>
-__device__ void fin_start(BScal *bs, const double (&t)[K], double tol2, int maxit, bool df = false)
+__device__ void fin_start(BScal *bs, const double *t, double tol2, int maxit, bool df = false)
 {
-    for (int c = 0; c < K; c++) {
+    const int c = threadIdx.x & 31;
+    int done = 1;
+    if (c < K) {
         CgScal &s = bs->c[c];
-        double ff = t[c];
+        const double ff = t[c];
+        // power of two nearest 1 / ||f||: the FP32 V-cycle sees r scaled by it
+        // (exact, and PCG is invariant under a scalar multiple of the
+        // preconditioner), which keeps tiny residuals inside FP32's range
+        const double nrm = sqrt(ff);
+        const double scale = (nrm > 0.0 && !nonfinite(nrm)) ? exp2(-rint(log2(nrm))) : 1.0;
+        const double s2 = df ? scale * scale : 1.0; // a power of two: exact
         s.ff = ff;
-        s.rr = ff;
-        s.thr = tol2 * ff;
+        s.rr = ff * s2;
+        s.thr = tol2 * ff * s2;
         s.maxit = maxit;
         s.iters = 0;
         s.k1 = 0;
         s.alpha = 0.0;
         s.beta = 0.0;
         s.rz = 0.0;
-        s.status = CG_RUNNING;
-        s.done = 0;
-        // power of two nearest 1 / ||f||: the FP32 V-cycle sees r scaled by it
-        // (exact, and PCG is invariant under a scalar multiple of the
-        // preconditioner), which keeps tiny residuals inside FP32's range
-        double nrm = sqrt(ff);
-        s.scale = (nrm > 0.0 && !nonfinite(nrm)) ? exp2(-rint(log2(nrm))) : 1.0;
+        s.ra = 0.0;
+        s.scale = scale;
         s.ahi = s.alo = s.bhi = s.blo = 0.f;
-        if (df) {
-            double s2 = s.scale * s.scale; // a power of two: exact
-            s.rr = ff * s2;
-            s.thr = tol2 * ff * s2;
-        }
-        if (nonfinite(ff)) {
-            s.status = CG_NUMERIC;
-            s.done = 1;
-        } else if (ff == 0.0) {
-            s.status = CG_CONVERGED;
-            s.done = 1;
-        }
+        s.status = nonfinite(ff) ? CG_NUMERIC : ff == 0.0 ? CG_CONVERGED : CG_RUNNING;
+        done = s.status != CG_RUNNING;
+        s.done = done;
     }
-    bs_all<K>(bs);
+    bs_all(bs, done);
 }
 
 // single-reduction PCG: gamma = (r, z), delta = (z, A z) -> alpha, beta
 template <int K>
-__device__ void fin_cg2(BScal *bs, const double (&t)[2 * K])
+__device__ void fin_cg2(BScal *bs, const double *t)
 {
-    for (int c = 0; c < K; c++) {
-        CgScal &s = bs->c[c];
-        if (s.done) continue;
-        double g = t[c], d = t[K + c];
-        if (!(g > 0.0) || !(d > 0.0)) {
-            s.status = (nonfinite(g) || nonfinite(d)) ? CG_NUMERIC : CG_INDEFINITE;
-            s.done = 1;
-            continue;
-        }
-        double beta = 0.0, alpha;
-        if (s.k1 == 0) {
-            alpha = g / d;
-        } else {
-            beta = g / s.rz;
-            double den = d - beta * g / s.alpha;
-            if (!(den > 0.0)) {
-                s.status = nonfinite(den) ? CG_NUMERIC : CG_INDEFINITE;
+    const int l = threadIdx.x & 31, c = min(l >> 1, K - 1);
+    CgScal &s = bs->c[c];
+    const double g = t[c];
+    const int k1 = s.k1;
+    int done = s.done;
+    double alpha, beta;
+    const int status = cg2_scalars(g, t[K + c], k1, s.rz, s.ra, alpha, beta);
+    __syncwarp(); // every lane has read its column's scalars
+    if (!done && l < 2 * K) {
+        if (status != CG_RUNNING) {
+            if (!(l & 1)) {
+                s.status = status;
                 s.done = 1;
-                continue;
             }
-            alpha = g / den;
+        } else if (!(l & 1)) {
+            s.rz = g;
+            s.ra = g * alpha;
+            s.alpha = alpha;
+            s.ahi = (float)alpha;
+            s.alo = (float)(alpha - (double)(float)alpha);
+            s.k1 = k1 + 1;
+        } else {
+            s.beta = beta;
+            s.bhi = (float)beta;
+            s.blo = (float)(beta - (double)(float)beta);
         }
-        s.rz = g;
-        s.alpha = alpha;
-        s.beta = beta;
-        s.ahi = (float)alpha;
-        s.alo = (float)(alpha - (double)s.ahi);
-        s.bhi = (float)beta;
-        s.blo = (float)(beta - (double)s.bhi);
-        s.k1 += 1;
     }
-    bs_all<K>(bs);
+    bs_all(bs, done || status != CG_RUNNING);
 }
 
 // r.r per column -> iteration count and stopping test
 template <int K>
-__device__ void fin_rr(BScal *bs, const double (&t)[K])
+__device__ void fin_rr(BScal *bs, const double *t)
 {
-    for (int c = 0; c < K; c++) {
+    const int c = threadIdx.x & 31;
+    int done = 1;
+    if (c < K) {
         CgScal &s = bs->c[c];
-        if (s.done) continue;
-        double rr = t[c];
-        s.rr = rr;
-        s.iters += 1;
-        s.total_iters += 1;
-        if (nonfinite(rr)) {
-            s.status = CG_NUMERIC;
-            s.done = 1;
-        } else if (rr <= s.thr) {
-            s.status = CG_CONVERGED;
-            s.done = 1;
-        } else if (s.iters >= s.maxit) {
-            s.status = CG_MAXIT;
-            s.done = 1;
+        done = s.done;
+        if (!done) {
+            const double rr = t[c];
+            s.rr = rr;
+            s.iters += 1;
+            s.total_iters += 1;
+            int status = CG_RUNNING;
+            if (!finite64(rr)) status = CG_NUMERIC;
+            else if (le64(rr, s.thr)) status = CG_CONVERGED;
+            else if (s.iters >= s.maxit) status = CG_MAXIT;
+            if (status != CG_RUNNING) {
+                s.status = status;
+                s.done = done = 1;
+            }
         }
     }
-    bs_all<K>(bs);
+    bs_all(bs, done);
 }
 
 // ------------------------------------------------------------------ CG kernels
@@ -608,7 +596,8 @@ __global__ void kb_cg_start(int n, const double *__restrict__ f, double *__restr
                             int maxit, double *partials, unsigned *ticket)
 {
     pdl_enter();
-    double v[K], tot[K];
+    double v[K];
+    const double *tot;
 #pragma unroll
     for (int c = 0; c < K; c++) v[c] = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -643,7 +632,8 @@ __global__ void kb_cg_spmv64(MatView<double> A, const double *__restrict__ z, co
     int row = my_row<TPR>();
     double sv[K];
     row_sum_k<double, TPR, K>(A, row, z, sv);
-    double a[2 * K], tot[2 * K];
+    double a[2 * K];
+    const double *tot;
 #pragma unroll
     for (int q = 0; q < 2 * K; q++) a[q] = 0.0;
     if (row < A.rows && row_leader<TPR>()) {
@@ -674,7 +664,8 @@ __global__ void kb_cg_update(int n, Z *z, const double *__restrict__ s, double *
     constexpr int KH = K / H;        // columns per thread
     pdl_enter();
     if (bs->all) return;
-    double v[K], tot[K];
+    double v[K];
+    const double *tot;
 #pragma unroll
     for (int c = 0; c < K; c++) v[c] = 0.0;
     const int64_t items = (int64_t)n * H;
@@ -690,7 +681,7 @@ __global__ void kb_cg_update(int n, Z *z, const double *__restrict__ s, double *
         al[c] = sc.alpha;
         be[c] = sc.beta;
         run[c] = !sc.done;
-        first[c] = sc.beta == 0.0;
+        first[c] = sc.k1 == 1;
     }
     double vh[KH];
 #pragma unroll
@@ -763,7 +754,8 @@ __global__ void kbd_norm(int n, const double *__restrict__ f, BScal *bs, double 
                          double *partials, unsigned *ticket)
 {
     pdl_enter();
-    double v[K], tot[K];
+    double v[K];
+    const double *tot;
 #pragma unroll
     for (int c = 0; c < K; c++) v[c] = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -808,7 +800,7 @@ __global__ void __launch_bounds__(TPB_K, 3) kbd_spmv(MatView<float> A, const flo
     DF sv[K];
     row_sum_df_k<float, TPR, K>(A, lo, row, z, sv);
     DF a[2 * K];
-    double tot[2 * K];
+    const double *tot;
 #pragma unroll
     for (int q = 0; q < 2 * K; q++) a[q] = DF{0.f, 0.f};
     if (row < A.rows && row_leader<TPR>()) {
@@ -914,7 +906,7 @@ __global__ void kbd_update(int n, float *z, const float *__restrict__ sh, const 
         }
     }
     DF v[K];
-    double tot[K];
+    const double *tot;
 #pragma unroll
     for (int c = 0; c < K; c++) v[c] = DF{0.f, 0.f};
 #pragma unroll
@@ -969,7 +961,6 @@ __global__ void __launch_bounds__(TPB_K) kbp_mass_cg(MatView<float> A, const flo
     for (int it = 0; it <= cap && !sb.all; it++) {
         // ---- s = A z, (r, z), (z, s)
         DF a[2 * K];
-        double tot[2 * K];
 #pragma unroll
         for (int q = 0; q < 2 * K; q++) a[q] = DF{0.f, 0.f};
         for (int base = blockIdx.x * blockDim.x; base < slots; base += stride) {
@@ -998,8 +989,8 @@ __global__ void __launch_bounds__(TPB_K) kbp_mass_cg(MatView<float> A, const flo
         }
         block_df_partials<2 * K>(a, p1, nb, blockIdx.x, st);
         if (!grid_sync(gb, nb)) return;
-        sum_df_partials<2 * K>(p1, nb, tot, st);
-        if (t == 0) fin_cg2<K>(&sb, tot);
+        sum_df_partials<2 * K>(p1, nb, st);
+        if (t < 32) fin_cg2<K>(&sb, st.tot);
         __syncthreads();
         // ---- p = z + beta p, q = s + beta q, x += alpha p, r -= alpha q, z = D^-1 r_hi, r.r
         const int64_t items = (int64_t)n * H;
@@ -1064,7 +1055,6 @@ __global__ void __launch_bounds__(TPB_K) kbp_mass_cg(MatView<float> A, const flo
             stk<KH>(z + o, zn);
         }
         DF v[K];
-        double rr[K];
 #pragma unroll
         for (int c = 0; c < K; c++) v[c] = DF{0.f, 0.f};
 #pragma unroll
@@ -1074,8 +1064,8 @@ __global__ void __launch_bounds__(TPB_K) kbp_mass_cg(MatView<float> A, const flo
         }
         block_df_partials<K, 2 * K>(v, p2, nb, blockIdx.x, st);
         if (!grid_sync(gb, nb)) return;
-        sum_df_partials<K, 2 * K>(p2, nb, rr, st);
-        if (t == 0) fin_rr<K>(&sb, rr);
+        sum_df_partials<K, 2 * K>(p2, nb, st);
+        if (t < 32) fin_rr<K>(&sb, st.tot);
         __syncthreads();
     }
     if (blockIdx.x == 0 && t == 0) *bs = sb;
@@ -1273,7 +1263,8 @@ __global__ void kb_dot(int n, const double *__restrict__ x, const double *__rest
                        double *partials, unsigned *ticket)
 {
     pdl_enter();
-    double v[K], tot[K];
+    double v[K];
+    const double *tot;
 #pragma unroll
     for (int c = 0; c < K; c++) v[c] = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1284,10 +1275,7 @@ __global__ void kb_dot(int n, const double *__restrict__ x, const double *__rest
 #pragma unroll
         for (int c = 0; c < K; c++) v[c] += xv[c] * yv[c];
     }
-    if (reduce_k<K>(v, partials, ticket, tot)) {
-#pragma unroll
-        for (int c = 0; c < K; c++) out[c] = tot[c];
-    }
+    if (reduce_k<K>(v, partials, ticket, tot) && threadIdx.x < K) out[threadIdx.x] = tot[threadIdx.x];
 }
 
 // column-major (leading dimension ld, nc columns) -> interleaved K columns,
@@ -1887,6 +1875,17 @@ struct Blk {
         const bool z32 = W.f32 != 0;
         std::function<int()> iter;
         const bool persist = z32 && W.pbar != nullptr;
+        if (!persist && mass_cluster_fits(C.Mu, z32)) { // one cluster per column
+            TRY(mass_cluster(p, C, z32, b, x, D.mbs->c, K, tol, maxit));
+            BScal h;
+            TRY(read_bscal(p, D.mbs, &h));
+            for (int c = 0; c < K; c++) {
+                p->c_mass += h.c[c].iters;
+                p->c_mass_lvl[l] += h.c[c].iters;
+                note_fail(W, c, col_status(h.c[c]));
+            }
+            return AMGH_OK;
+        }
         if (z32) {
             TRY(df_start(p, n, b, D.mx, D.mr, (float *)D.mz, (const float *)C.mu_invdiag32, D.mbs, D.red, tol,
                          maxit));

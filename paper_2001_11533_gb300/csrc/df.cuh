@@ -131,8 +131,8 @@ __device__ __forceinline__ DF df_warp_sum(DF v)
 // Sum over the grid of NV double-float values per thread: warp butterflies,
 // then warp 0 of each block, then the last block to finish sums the blocks'
 // partials (double-float, two FP32 halves in each 8-byte slot of partials,
-// [NV][gridDim.x]) in fixed order.  Returns true in thread 0 of that block,
-// with the sums (as FP64) in tot.  Every FP64 instruction costs ~64 FP32
+// [NV][gridDim.x]) in fixed order.  Returns true in the first warp of that
+// block, with the sums (as FP64) in tot.  Every FP64 instruction costs ~64 FP32
 // issue slots on GB300, so the tree stays on the FP32 pipe.
 template <int NV>
 __device__ bool reduce_df_last_block(const DF (&val)[NV], double *partials, unsigned *ticket, double (&tot)[NV])
@@ -185,5 +185,5 @@ __device__ bool reduce_df_last_block(const DF (&val)[NV], double *partials, unsi
         }
         if (l == 0) *ticket = 0u;
     }
-    return threadIdx.x == 0;
+    return threadIdx.x < 32;
 }

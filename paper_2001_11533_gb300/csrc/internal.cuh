@@ -216,7 +216,7 @@ struct CgScal {
     int total_iters;
     int k1; // single-reduction CG: number of alpha/beta updates so far
     float ahi, alo, bhi, blo; // alpha and beta as double-float (double-float CG)
-    int pad[2];
+    double ra;                // rz alpha of the last alpha/beta update (cg2_scalars)
 };
 
 enum { CG_RUNNING = 0, CG_CONVERGED = 1, CG_INDEFINITE = 2, CG_NUMERIC = 3, CG_MAXIT = 4 };

@@ -49,8 +49,8 @@ __device__ __forceinline__ double block_sum(double v, double *sh32)
 }
 
 // Last-block finalisation of a two-stage reduction with NV values per block.
-// Returns true in thread 0 of the block that finished last; `tot` then holds
-// the fixed-order sums of all partials.  partials layout: [NV][gridDim.x].
+// Returns true in the first warp of the block that finished last; `tot` then
+// holds the fixed-order sums of all partials.  partials layout: [NV][gridDim.x].
 template <int NV>
 __device__ bool reduce_last_block(const double (&val)[NV], double *partials, unsigned *ticket,
                                   double (&tot)[NV])
@@ -101,7 +101,7 @@ __device__ bool reduce_last_block(const double (&val)[NV], double *partials, uns
         }
     }
     if (threadIdx.x == 0) *ticket = 0u;
-    return threadIdx.x == 0;
+    return threadIdx.x < 32;
 }
 
 // Order of non-negative FP64 numbers by their bits: an FP64 comparison, like
@@ -121,8 +121,9 @@ __device__ __forceinline__ bool le64(double x, double y) // x <= y, both >= 0
 // g = (r, z), d = (z, A z) and, from the step before (k1 > 0), rz = g' and
 // ra = g' alpha':
 //   beta = g / g',  alpha = g / (d - beta g / alpha') = g ra / (d ra - g^2).
-// Called by all lanes of one warp with the same arguments; all get the result.
-// An FP64 division takes ten dependent FP64 instructions, so the two divisions
+// Called by all lanes of a warp, lanes 2c and 2c + 1 with the scalars of loop c
+// (the same for all lanes where there is one loop); both get the result.  An
+// FP64 division takes ten dependent FP64 instructions, so the two divisions
 // are made by two lanes of one instruction sequence (in the textbook order
 // three divisions follow each other).  The products are formed on g and ra
 // scaled by the power of two of g, so that no square over- or underflows where
@@ -140,8 +141,9 @@ __device__ __forceinline__ int cg2_scalars(double g, double d, int k1, double rz
     }
     const bool second = threadIdx.x & 1;
     const double quo = (second ? g : num) / (second ? rz : den);
-    alpha = __shfl_sync(0xffffffffu, quo, 0);
-    beta = __shfl_sync(0xffffffffu, quo, 1);
+    const double other = __shfl_xor_sync(0xffffffffu, quo, 1);
+    alpha = second ? other : quo;
+    beta = second ? quo : other;
     if (!k1) beta = 0.0;
     if (pos64(g) && pos64(d) && pos64(den)) return CG_RUNNING;
     return finite64(g) && finite64(d) && finite64(den) ? CG_INDEFINITE : CG_NUMERIC;
