@@ -1824,11 +1824,13 @@ struct Blk {
         int maxit = p->sopts.inner_max_iter;
         const bool f32 = sizeof(T) == sizeof(float);
         T *z = (T *)B.z;
+        // the V-cycle's input; the bodies below refer to it for as long as
+        // run_loop captures them
+        const T *vin = sizeof(T) == sizeof(float) ? (const T *)hi(B.r) : (const T *)B.r;
         std::function<int()> start, iter;
         if constexpr (sizeof(T) == sizeof(float)) {
             // double-float CG; the FP32 V-cycle reads r's hi half
             TRY(df_start(p, n, f, B.x, B.r, (float *)nullptr, (const float *)nullptr, B.bs, B.red, tol, maxit));
-            const T *vin = (const T *)hi(B.r);
             start = [&]() { return vcyc(p, l, vin, z, B.bs); };
             iter = [&]() {
                 TRY(df_iter(p, S.A, (float *)z, B.r, B.s, B.pv, B.q, B.x, (const float *)nullptr, B.bs, B.red));
@@ -1839,7 +1841,6 @@ struct Blk {
                        (double *)nullptr, (const double *)nullptr, B.bs, tol * tol, maxit, B.red.partials,
                        B.red.ticket);
             LAUNCH_CHECK();
-            const T *vin = (const T *)B.r;
             start = [&]() { return vcyc(p, l, vin, z, B.bs); };
             iter = [&]() {
                 TRY(cg_spmv<T>(p, S.A, z, B.r, B.s, B.bs, B.red));
