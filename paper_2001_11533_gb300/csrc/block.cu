@@ -1324,6 +1324,8 @@ __global__ void kb_gather_state(int m, int nc, const double *__restrict__ yd, in
 struct BGraph {
     cudaGraphExec_t start = nullptr, iter = nullptr;
     int ns = 0, ni = 0;
+    cudaGraphExec_t run = nullptr; // CG_RUN iterations, as CgGraph
+    int64_t ran = 0;
 };
 
 struct BState {
@@ -1369,6 +1371,7 @@ static void free_bgraph(BGraph &g)
 {
     if (g.start) cudaGraphExecDestroy(g.start);
     if (g.iter) cudaGraphExecDestroy(g.iter);
+    if (g.run) cudaGraphExecDestroy(g.run);
     g = BGraph();
 }
 
@@ -1792,11 +1795,24 @@ struct Blk {
             if (gr) TRY(graph_replay(p, g.start, g.ns));
             else TRY(start());
         }
-        int chunk = *hint > 1 ? (*hint * 7) / 8 : 1;
+        int chunk = *hint > 1 ? *hint : 1;
         int enq = 0;
         BScal h;
         for (;;) {
-            for (int c = 0; c < chunk; c++) {
+            if (gr && !g.run && chunk >= CG_RUN && g.ran >= CG_RUN_AFTER) {
+                int nodes = 0;
+                TRY(graph_capture(
+                    p,
+                    [&]() -> int {
+                        for (int c = 0; c < CG_RUN; c++) TRY(iter());
+                        return AMGH_OK;
+                    },
+                    &g.run, &nodes));
+            }
+            g.ran += chunk;
+            int left = chunk;
+            for (; gr && g.run && left >= CG_RUN; left -= CG_RUN) TRY(graph_replay(p, g.run, CG_RUN * g.ni));
+            for (; left > 0; left--) {
                 if (gr) TRY(graph_replay(p, g.iter, g.ni));
                 else TRY(iter());
             }

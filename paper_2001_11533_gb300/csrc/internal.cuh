@@ -228,10 +228,18 @@ enum { CG_RUNNING = 0, CG_CONVERGED = 1, CG_INDEFINITE = 2, CG_NUMERIC = 3, CG_M
 struct CgGraph {
     cudaGraphExec_t start = nullptr, iter = nullptr;
     int nodes_start = 0, nodes_iter = 0;
+    // CG_RUN iterations in one graph, captured once `ran` single ones have paid
+    // for it: replays of one graph after another leave a gap (no programmatic
+    // launch across graphs), iterations inside one do not
+    cudaGraphExec_t run = nullptr;
+    int64_t ran = 0;
     // algorithmic bytes of one replay, and of the iteration's V-cycle alone
     // (skipped in the iteration that converges)
     double bytes_start = 0.0, bytes_iter = 0.0, bytes_vc = 0.0;
 };
+
+#define CG_RUN 4
+#define CG_RUN_AFTER 24
 
 struct StateLevel {
     DevCsr A, My, S, St; // S: rows m_l, cols m_{l+1}; St = S^T

@@ -292,10 +292,35 @@ static int replay(amgh_problem *p, cudaGraphExec_t ex, int nodes)
     return AMGH_OK;
 }
 
+// `count` iterations of a CG loop by graph replay, CG_RUN at a time where that
+// graph exists.  A captured graph costs a few hundred microseconds, a gap
+// between two replays about 2.5: the CG_RUN graph is made once the loop has run
+// CG_RUN_AFTER iterations (65^2 mixed solve 18.2 -> 17.0 ms, preconditioner on
+// 201^2 6.35 -> 5.78 ms; eight at a time gains nothing more).
+template <typename F>
+static int replay_iters(amgh_problem *p, CgGraph &g, int count, F body)
+{
+    if (!g.run && count >= CG_RUN && g.ran >= CG_RUN_AFTER) {
+        int nodes = 0;
+        TRY(capture(
+            p,
+            [&] {
+                for (int c = 0; c < CG_RUN; c++) TRY(body());
+                return (int)AMGH_OK;
+            },
+            &g.run, &nodes));
+    }
+    g.ran += count;
+    for (; g.run && count >= CG_RUN; count -= CG_RUN) TRY(replay(p, g.run, CG_RUN * g.nodes_iter));
+    for (; count > 0; count--) TRY(replay(p, g.iter, g.nodes_iter));
+    return AMGH_OK;
+}
+
 static void free_graph(CgGraph &g)
 {
     if (g.start) cudaGraphExecDestroy(g.start);
     if (g.iter) cudaGraphExecDestroy(g.iter);
+    if (g.run) cudaGraphExecDestroy(g.run);
     g = CgGraph();
 }
 
@@ -424,17 +449,19 @@ static int pcg_run(amgh_problem *p, int l, int mode, const void *f, double tol, 
         TRY(cg_body_start(p, l, mode));
     }
     int *hint = mode == 1 ? &p->chunk_hint32[l] : &p->chunk_hint[l];
-    // first chunk: most of the previous solve's count (replays past convergence are no-ops)
-    int chunk = *hint > 1 ? (*hint * 7) / 8 : 1;
+    // first chunk: the previous solve's count.  A replay past convergence is
+    // ~0.7 us a kernel (about 15 us), a read of the flag leaves the GPU idle
+    // for about 10 us, and counts rarely differ by more than one or two
+    int chunk = *hint > 1 ? *hint : 1;
     int enq = 0, prev_iters = 0;
     CgScal h;
     std::vector<size_t> it_mark, vc_mark; // direct launches: timings of each enqueued iteration
     for (;;) {
         it_mark.clear();
         vc_mark.clear();
-        for (int c = 0; c < chunk; c++) {
-            if (gr) TRY(replay(p, g.iter, g.nodes_iter));
-            else {
+        if (gr) TRY(replay_iters(p, g, chunk, [&] { return cg_body_iter(p, l, mode); }));
+        for (int c = 0; !gr && c < chunk; c++) {
+            {
                 double b = 0.0;
                 it_mark.push_back(p->timer.ev.size());
                 {
@@ -557,15 +584,15 @@ int mass_solve(amgh_problem *p, int l, const double *b, double *x, int64_t *iter
     };
     if (gr && !g.iter) TRY(capture(p, body, &g.iter, &g.nodes_iter, &g.bytes_iter));
     double b_iter = g.bytes_iter;
-    int chunk = p->mchunk_hint[l] > 1 ? (p->mchunk_hint[l] * 7) / 8 : 1;
+    int chunk = p->mchunk_hint[l] > 1 ? p->mchunk_hint[l] : 1;
     int enq = 0, prev_iters = 0;
     CgScal h;
     std::vector<size_t> it_mark;
     for (;;) {
         it_mark.clear();
-        for (int c = 0; c < chunk; c++) {
-            if (gr) TRY(replay(p, g.iter, g.nodes_iter));
-            else {
+        if (gr) TRY(replay_iters(p, g, chunk, body));
+        for (int c = 0; !gr && c < chunk; c++) {
+            {
                 double b = 0.0;
                 it_mark.push_back(p->timer.ev.size());
                 {
