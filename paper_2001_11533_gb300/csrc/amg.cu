@@ -1296,12 +1296,14 @@ int galerkin(amgh_problem *p, Arena &ar, const DevCsr &rt, const DevCsr &a, cons
 
 // c1 = rt a1 pm and c2 = rt a2 pm for a1, a2 with one sparsity pattern (A and
 // M_y, or K_N and M_u): both products share their hashing and the result's
-// pattern (c2 uses c1's row pointers and columns); both made exactly symmetric
+// pattern (c2 uses c1's row pointers and columns); both made exactly symmetric.
+// keep: where the first product a1 pm (canonical CSR) is left instead of freed
 int galerkin_pair(amgh_problem *p, Arena &ar, const DevCsr &rt, const DevCsr &a1, const DevCsr &a2,
-                  const DevCsr &pm, DevCsr &c1, DevCsr &c2)
+                  const DevCsr &pm, DevCsr &c1, DevCsr &c2, KeptProduct *keep)
 {
     if (a1.rows != a2.rows || a1.nnz != a2.nnz) return AMGH_ERR_INVALID_ARG;
-    Arena tmp;
+    Arena own;
+    Arena &tmp = keep ? keep->ar : own;
     DevCsr ap;
     double *apv[2] = {nullptr, nullptr};
     const double *av[2] = {a1.v, a2.v}, *pv[2] = {pm.v, pm.v};
@@ -1321,7 +1323,8 @@ int galerkin_pair(amgh_problem *p, Arena &ar, const DevCsr &rt, const DevCsr &a1
             c2.v = cv[1];
         }
     }
-    tmp.free_all();
+    if (keep) keep->m = ap;
+    own.free_all();
     if (st) return st;
     TRY(symmetrize_upper(p, c1));
     TRY(symmetrize_upper(p, c2));

@@ -367,8 +367,9 @@ static int setup_impl(amgh_problem *p)
     TRY(extract_sub(ar, p->Mfull, p->state_of_vertex, p->m, nullptr, p->n, C0.Myu, s));
     TRY(extract_sub(ar, p->Kfull, nullptr, p->n, nullptr, p->n, C0.KN, s));
     TRY(extract_sub(ar, p->Mfull, nullptr, p->n, nullptr, p->n, C0.Mu, s));
+    KeptProduct as[AMGH_MAXL]; // A_l S_l where the transfers use it, freed once they are laid out
     if (o.geometric) {
-        TRY(geometric_hierarchy(p));
+        TRY(geometric_hierarchy(p, as));
         goto hierarchies_done;
     }
     {
@@ -386,7 +387,8 @@ static int setup_impl(amgh_problem *p)
         S.nagg = nagg;
         TRY(amg_prolongator(p, ar, S.A, S.agg, nagg, o.smooth_prolongator, S.S));
         TRY(csr_transpose(ar, S.S, S.St, s));
-        TRY(galerkin_pair(p, ar, S.St, S.A, S.My, S.S, p->sl[l + 1].A, p->sl[l + 1].My));
+        TRY(galerkin_pair(p, ar, S.St, S.A, S.My, S.S, p->sl[l + 1].A, p->sl[l + 1].My,
+                          transfer_fits(p, l) ? &as[l] : nullptr));
         p->Ls = l + 2;
         th = th * 0.5;
     }
@@ -423,6 +425,10 @@ hierarchies_done:
         if (l + 1 < p->Ls) {
             TRY(prepare_operator(ar, S.S, s));
             TRY(prepare_operator(ar, S.St, s));
+            if (transfer_fits(p, l)) {
+                TRY(transfer_setup(p, ar, S, as[l].m));
+                as[l].ar.free_all();
+            }
         }
         TRY(ar.alloc(&S.invd, S.A.rows));
         TRY(ar.alloc(&S.invd32, S.A.rows));

@@ -47,9 +47,11 @@ struct GridScope {
 
 struct FusedLevel {
     MatView<float> A, St, S; // St: rows of level l+1; S: rows of level l
+    MatView<float> dn, up;   // pair matrices with the rows of St and S (transfer.cu)
+    const float *dn_s, *up_s;
     const float *invd;
     float *b, *x, *x2, *d, *r;
-    int n;
+    int n, paired;
 };
 
 struct FusedCycle {
@@ -141,6 +143,55 @@ __device__ void ph_prolong(const FusedLevel &L, const float *e, float *x, int g,
     });
 }
 
+// b_c = S^T b - (A S)^T x; with first, also the coarse level's first smoother
+// step d_c = x2_c = c0 D_c^-1 b_c
+template <int TPR>
+__device__ void ph_restrict_pair(const FusedLevel &L, const FusedLevel &C, const float *b, const float *x, int first,
+                            float c0, int g, int T)
+{
+    sweep_rows<TPR>(C.n, g, T, [&](int i) {
+        RowPrePair<float> pre;
+        row_prefetch_pair<float, TPR>(L.dn, L.dn_s, i, pre);
+        float bv = row_restrict_pair<float, TPR>(
+            L.dn, L.dn_s, i, pre, [&](int c) { return __ldcg(b + c); }, [&](int c) { return __ldcg(x + c); });
+        if (i < C.n && row_leader<TPR>()) {
+            C.b[i] = bv;
+            if (first) {
+                float v = cheb_first_point(bv, C.invd[i], c0);
+                C.d[i] = v;
+                C.x2[i] = v;
+            }
+        }
+    });
+}
+
+// xn = x + S e + d, d = c D^-1 (b - A x - (A S) e)
+template <int TPR>
+__device__ void ph_prolong_pair(const FusedLevel &L, const float *b, const float *x, const float *e, float *xn, float c,
+                           int g, int T)
+{
+    sweep_rows<TPR>(L.n, g, T, [&](int r) {
+        bool lead = r < L.n && row_leader<TPR>();
+        float br = 0.f, ir = 0.f, xr = 0.f;
+        if (lead) {
+            br = __ldcg(b + r);
+            ir = L.invd[r];
+            xr = __ldcg(x + r);
+        }
+        float ax = row_sum<float, TPR>(L.A, r, [&](int j) { return __ldcg(x + j); });
+        RowPrePair<float> pre;
+        row_prefetch_pair<float, TPR>(L.up, L.up_s, r, pre);
+        float ase, se;
+        row_prolong_pair<float, TPR>(L.up, L.up_s, r, pre, [&](int j) { return __ldcg(e + j); }, ase, se);
+        if (lead) {
+            float dn, xv;
+            prolong_point(br, ax, ase, se, ir, xr, c, dn, xv);
+            L.d[r] = dn;
+            xn[r] = xv;
+        }
+    });
+}
+
 template <typename Scope>
 __device__ __forceinline__ void vcycle_body(const FusedCycle *__restrict__ fc, const float *b0, float *x0,
                                             int preinit, int g, int T, Scope &cl)
@@ -171,14 +222,20 @@ __device__ __forceinline__ void vcycle_body(const FusedCycle *__restrict__ fc, c
             c = nx;
             nx = t;
         }
-#define CALL(K) ph_residual<K>(L, b, c, g, T)
-        TPR_DISPATCH(L.A.tpr, CALL)
-#undef CALL
-        if (!cl.sync()) return;
         const FusedLevel &C = fc->lv[l + 1];
-#define CALL(K) ph_restrict<K>(L, C, l + 1 < last, fc->cr[0], g, T)
-        TPR_DISPATCH(L.St.tpr, CALL)
+        if (L.paired) {
+#define CALL(K) ph_restrict_pair<K>(L, C, b, c, l + 1 < last, fc->cr[0], g, T)
+            TPR_DISPATCH(L.dn.tpr, CALL)
 #undef CALL
+        } else {
+#define CALL(K) ph_residual<K>(L, b, c, g, T)
+            TPR_DISPATCH(L.A.tpr, CALL)
+#undef CALL
+            if (!cl.sync()) return;
+#define CALL(K) ph_restrict<K>(L, C, l + 1 < last, fc->cr[0], g, T)
+            TPR_DISPATCH(L.St.tpr, CALL)
+#undef CALL
+        }
         if (!cl.sync()) return;
         cur[l] = c;
         nxt[l] = nx;
@@ -200,11 +257,22 @@ __device__ __forceinline__ void vcycle_body(const FusedCycle *__restrict__ fc, c
         const float *b = l == c0 ? b0 : L.b;
         float *x = l == c0 ? x0 : L.x;
         float *c = cur[l], *nx = nxt[l];
-#define CALL(K) ph_prolong<K>(L, fc->lv[l + 1].x, c, g, T)
-        TPR_DISPATCH(L.S.tpr, CALL)
+        int s0 = 0;
+        if (L.paired) { // with the first post-smoothing step
+#define CALL(K) ph_prolong_pair<K>(L, b, c, fc->lv[l + 1].x, nx, fc->cr[0], g, T)
+            TPR_DISPATCH(L.A.tpr, CALL)
 #undef CALL
+            float *t = c;
+            c = nx;
+            nx = t;
+            s0 = 1;
+        } else {
+#define CALL(K) ph_prolong<K>(L, fc->lv[l + 1].x, c, g, T)
+            TPR_DISPATCH(L.S.tpr, CALL)
+#undef CALL
+        }
         if (!cl.sync()) return;
-        for (int s = 0; s < ns; s++) {
+        for (int s = s0; s < ns; s++) {
 #define CALL(K) ph_cheb<K>(L, b, c, nx, s == 0 ? 0.f : fc->cd[s], fc->cr[s], g, T)
             TPR_DISPATCH(L.A.tpr, CALL)
 #undef CALL
@@ -286,6 +354,13 @@ int fused_setup(amgh_problem *p)
         if (l < h.last) {
             L.St = view<float>(S.St);
             L.S = view<float>(S.S);
+            L.paired = S.paired;
+            if (S.paired) {
+                L.dn = view<float>(S.down.m);
+                L.up = view<float>(S.up.m);
+                L.dn_s = S.down.s;
+                L.up_s = S.up.s;
+            }
         }
         L.invd = S.invd32;
         L.b = S.fb;

@@ -109,7 +109,7 @@ __global__ void k_geo_interp(int N, int *__restrict__ rp, int *__restrict__ ci, 
     }
 }
 
-int geometric_hierarchy(amgh_problem *p)
+int geometric_hierarchy(amgh_problem *p, KeptProduct *as)
 {
     const amgh_amg_opts &o = p->aopts;
     cudaStream_t s = p->stream;
@@ -158,7 +158,8 @@ int geometric_hierarchy(amgh_problem *p)
         LAUNCH_CHECK();
         TRY(extract_sub(ar, P, fmap, (N - 2) * (N - 2), cmap, (Nc - 2) * (Nc - 2), S.S, s));
         TRY(csr_transpose(ar, S.S, S.St, s));
-        TRY(galerkin_pair(p, ar, S.St, S.A, S.My, S.S, p->sl[l + 1].A, p->sl[l + 1].My));
+        TRY(galerkin_pair(p, ar, S.St, S.A, S.My, S.S, p->sl[l + 1].A, p->sl[l + 1].My,
+                          transfer_fits(p, l) ? &as[l] : nullptr));
         TRY(csr_transpose(ar, P, C.Pt, s));
         TRY(galerkin_pair(p, ar, C.Pt, C.KN, C.Mu, P, p->cl[l + 1].KN, p->cl[l + 1].Mu));
         S.nagg = (Nc - 2) * (Nc - 2);

@@ -198,6 +198,13 @@ struct DevCsr {
     int nnz_solve = -1;
 };
 
+// Two coefficients per pair (i, k) in one layout (transfer.cu): m holds A S (or
+// its transpose), s the matching FP32 entries of S (S^T)
+struct PairMat {
+    DevCsr m;
+    float *s = nullptr;
+};
+
 // ------------------------------------------------------------------ reductions
 // Deterministic two-stage reductions: every block writes a partial, the last
 // block to finish (atomic ticket) sums the partials in fixed order and runs a
@@ -243,6 +250,8 @@ struct CgGraph {
 
 struct StateLevel {
     DevCsr A, My, S, St; // S: rows m_l, cols m_{l+1}; St = S^T
+    PairMat up, down;    // A S with S (rows m_l), and transposed (rows m_{l+1})
+    bool paired = false; // built (transfer.cu)
     double *invd = nullptr;   // 1 / l1 row sums
     float *invd32 = nullptr;
     int *agg = nullptr;
@@ -432,6 +441,8 @@ void mis_set_round_cap(int cap);
 void prol_set_row_cap(int cap);
 // b = (float)a
 int to_f32(amgh_problem *p, const double *a, int64_t n, float *b);
+// the layout itself, without leaving out exact zeros
+int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr);
 // build a.lo32 (after prepare_operator)
 int build_lo_parts(Arena &ar, DevCsr &a, cudaStream_t s);
 int csr_transpose(Arena &ar, const DevCsr &a, DevCsr &t, cudaStream_t s);
@@ -519,6 +530,15 @@ int vec_dot(amgh_problem *p, RedSlot &red, int n, const double *x, const double 
 int scatter_state(amgh_problem *p, int m, const int *vertex_of_state, const double *ys,
                   double *full, double scale_add_beta_u, const double *u);
 
+// ------------------------------------------------------------------ transfer.cu
+// whether level l's FP32 transfers are fused with the products beside them
+bool transfer_fits(const amgh_problem *p, int l);
+int transfer_setup(amgh_problem *p, Arena &ar, StateLevel &S, const DevCsr &as);
+int restrict_pair(amgh_problem *p, const StateLevel &S, const float *b, const float *x, float *bc,
+                  const float *invd_c, float *d_c, float *x_c, double c0, const int *skip);
+int prolong_pair(amgh_problem *p, const StateLevel &S, const float *b, const float *x, const float *e, float *d,
+                 float *xn, double c, const int *skip);
+
 // ------------------------------------------------------------------ mass.cu
 // whether the mass CG of this level runs as one cluster launch; the launch:
 // cols right sides interleaved (element i of column c at i * cols + c), the
@@ -532,6 +552,15 @@ int assemble_full(amgh_problem *p);
 int extract_sub(Arena &ar, const DevCsr &a, const int *rmap, int nr, const int *cmap, int nc,
                 DevCsr &out, cudaStream_t s);
 
+// a product of the Galerkin setup kept for transfer.cu, with its memory
+struct KeptProduct {
+    DevCsr m;
+    Arena ar;
+    KeptProduct() = default;
+    KeptProduct(const KeptProduct &) = delete;
+    ~KeptProduct() { ar.free_all(); }
+};
+
 // ------------------------------------------------------------------ amg.cu
 int amg_aggregate(amgh_problem *p, const DevCsr &a, double theta2, int *agg, int *nagg);
 // aggressive first-level aggregation: the aggregates of a, aggregated once
@@ -539,7 +568,7 @@ int amg_aggregate(amgh_problem *p, const DevCsr &a, double theta2, int *agg, int
 int amg_aggregate_aggressive(amgh_problem *p, const DevCsr &a, double theta2, int *agg, int *nagg);
 // the geometric hierarchy of a structured N x N square grid (aopts.geometric):
 // fills S, St, P, Pt and the Galerkin A, M_y, K_N, M_u of every level, Ls = Lc
-int geometric_hierarchy(amgh_problem *p);
+int geometric_hierarchy(amgh_problem *p, KeptProduct *as);
 int amg_prolongator(amgh_problem *p, Arena &ar, const DevCsr &a, const int *agg, int nagg,
                     int smooth, DevCsr &s);
 int spgemm(amgh_problem *p, Arena &ar, const DevCsr &a, const DevCsr &b, DevCsr &c);
@@ -548,8 +577,9 @@ int galerkin(amgh_problem *p, Arena &ar, const DevCsr &rt, const DevCsr &a, cons
              int symmetric, DevCsr &c);
 // the same Galerkin product for two matrices with one sparsity pattern, in one
 // pass (results share row pointers and columns)
+// (keep: receives a1 pm and the memory that holds it)
 int galerkin_pair(amgh_problem *p, Arena &ar, const DevCsr &rt, const DevCsr &a1, const DevCsr &a2,
-                  const DevCsr &pm, DevCsr &c1, DevCsr &c2);
+                  const DevCsr &pm, DevCsr &c1, DevCsr &c2, KeptProduct *keep = nullptr);
 int l1_invdiag(amgh_problem *p, const DevCsr &a, double *invd, float *invd32);
 int diag_inv(amgh_problem *p, const DevCsr &a, double *invd);
 

@@ -190,29 +190,36 @@ static int vcyc(amgh_problem *p, int l, const T *b, T *x, const int *skip, int p
         cur = nxt;
         nxt = t;
     }
-    // coarse-grid correction
-    if (mf) TRY(kuhn_residual(p, (const float *)b, (const float *)cur, (float *)r, skip));
-    else TRY(residual<T>(p, S.A, b, cur, r, skip, timed));
     StateLevel &Sc = p->sl[l + 1];
     T *bc = VBuf<T>::b(Sc), *xc = VBuf<T>::x(Sc);
-    if (l + 1 < p->Ls - 1) {
-        TRY(restrict_first<T>(p, S.St, r, bc, VBuf<T>::invd(Sc), VBuf<T>::d(Sc), VBuf<T>::x2(Sc), p->cr[0], skip));
-        TRY(vcyc<T>(p, l + 1, bc, xc, skip, 1));
+    const int smooths = l + 1 < p->Ls - 1; // the coarse level has smoother steps
+    int s0 = 0;                            // post-smoothing steps already taken
+    if (!mf && S.paired && sizeof(T) == sizeof(float)) {
+        // coarse-grid correction and the first post-smoothing step (transfer.cu)
+        TRY(restrict_pair(p, S, (const float *)b, (const float *)cur, (float *)bc, Sc.invd32,
+                          smooths ? Sc.fd : nullptr, Sc.fx2, p->cr[0], skip));
+        TRY(vcyc<T>(p, l + 1, bc, xc, skip, smooths));
+        TRY(prolong_pair(p, S, (const float *)b, (const float *)cur, (const float *)xc, (float *)d, (float *)nxt,
+                         p->cr[0], skip));
+        std::swap(cur, nxt);
+        s0 = 1;
     } else {
-        TRY(spmv_t<T>(p, S.St, r, bc, skip, l == 0 ? KC_RESTRICT0 : KC_RESTRICT));
-        TRY(vcyc<T>(p, l + 1, bc, xc, skip));
+        if (mf) TRY(kuhn_residual(p, (const float *)b, (const float *)cur, (float *)r, skip));
+        else TRY(residual<T>(p, S.A, b, cur, r, skip, timed));
+        if (smooths)
+            TRY(restrict_first<T>(p, S.St, r, bc, VBuf<T>::invd(Sc), VBuf<T>::d(Sc), VBuf<T>::x2(Sc), p->cr[0], skip));
+        else TRY(spmv_t<T>(p, S.St, r, bc, skip, l == 0 ? KC_RESTRICT0 : KC_RESTRICT));
+        TRY(vcyc<T>(p, l + 1, bc, xc, skip, smooths));
+        TRY(prolong_add<T>(p, S.S, xc, cur, skip));
     }
-    TRY(prolong_add<T>(p, S.S, xc, cur, skip));
     // post-smoothing with the same polynomial
-    for (int s = 0; s < p->nsteps; s++) {
+    for (int s = s0; s < p->nsteps; s++) {
         if (mf)
             TRY(kuhn_cheb_step(p, (const float *)invd, (const float *)b, (const float *)cur, (float *)d,
                                (float *)nxt, s == 0 ? 0.0 : p->cd[s], p->cr[s], skip));
         else
             TRY(cheb_step<T>(p, S.A, invd, b, cur, d, nxt, s == 0 ? 0.0 : p->cd[s], p->cr[s], skip, timed));
-        T *t = cur;
-        cur = nxt;
-        nxt = t;
+        std::swap(cur, nxt);
     }
     if (cur != x) {
         timer_begin(p, KC_VEC);
@@ -232,6 +239,13 @@ double vcycle_bytes(const amgh_problem *p, int l, int vb)
     if (l == p->Ls - 1) return vb == 4 ? 4.0 * n * p->Acoarse.ld32 + 8.0 * n : 8.0 * n * n + 2.0 * vb * n;
     const double step = spmv_bytes(S.A, vb) + 4.0 * vb * n;
     double b = 4.0 * vb * n + (p->nsteps - 1) * step;                 // pre-smoothing from zero
+    if (vb == 4 && S.paired) {
+        const DevCsr &dn = S.down.m, &up = S.up.m;
+        b += spmv_bytes(dn, vb) + vb * ((double)dn.nnz + n + 3.0 * dn.rows);     // restriction (+ first coarse step)
+        b += vcycle_bytes(p, l + 1, vb);
+        b += spmv_bytes(S.A, vb) + spmv_bytes(up, vb) + vb * (up.nnz + 2.0 * n); // prolongation + first step
+        return b + (p->nsteps - 1) * step;                                       // post-smoothing
+    }
     b += spmv_bytes(S.A, vb) + vb * n;                                 // residual
     b += spmv_bytes(S.St, vb) + 3.0 * vb * S.St.rows;                  // restriction (+ first coarse step)
     b += vcycle_bytes(p, l + 1, vb);

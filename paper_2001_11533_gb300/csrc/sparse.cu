@@ -325,8 +325,6 @@ __global__ void k_drop_zeros(int rows, const int *__restrict__ rp, const int *__
         }
 }
 
-static int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr);
-
 // Solve-phase layout of a.  Entries whose value is exactly zero (the P1
 // stiffness of the Kuhn cube stores 8 of its 15 entries per row as exact
 // zeros) are left out of the SELL copy: a zero term adds nothing to any row
@@ -378,7 +376,7 @@ int prepare_operator(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
     return prepare_layout(ar, a, s, force_tpr);
 }
 
-static int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
+int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
 {
     double avg = a.rows > 0 ? (double)a.nnz / a.rows : 0.0;
     int longest = 0;

@@ -160,6 +160,142 @@ __device__ __forceinline__ T row_sum(const MatView<T> &m, int row, F xf)
     return row_sum_pre<T, TPR>(m, row, p, xf);
 }
 
+// ---- point-wise V-cycle arithmetic with explicit rounding, shared by the
+// level-by-level kernels and the fused coarse cycle so both give the same bits
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// Chebyshev step at one row: d' = c_d d + c_r D^-1 (b - A x), x' = x + d'
+template <typename T>
+__device__ __forceinline__ void cheb_point(T br, T ax, T ir, T dr, T xr, T cdv, T crv, T &dn, T &xn)
+{
+    T res = rmul(rsub(br, ax), ir);
+    dn = rfma(cdv, dr, rmul(crv, res));
+    xn = radd(xr, dn);
+}
+
+// first step from zero: c D^-1 b
+template <typename T>
+__device__ __forceinline__ T cheb_first_point(T br, T ir, T c)
+{
+    return rmul(c, rmul(br, ir));
+}
+
+// prolongation with the first post-smoothing step (transfer.cu): d = c D^-1
+// (b - A x - (A S) e), x' = x + S e + d
+template <typename T>
+__device__ __forceinline__ void prolong_point(T br, T ax, T ase, T se, T ir, T xr, T c, T &dn, T &xn)
+{
+    dn = rmul(c, rmul(rsub(rsub(br, ax), ase), ir));
+    xn = radd(radd(xr, se), dn);
+}
+
+// A row of a pair matrix (transfer.cu): entries of A S with the matching
+// entries of S beside them
+template <typename T>
+struct RowPrePair {
+    RowPre<T> h;
+    T ss[ROW_UNROLL];
+};
+
+template <typename T, int TPR>
+__device__ __forceinline__ void row_load_pair(const MatView<T> &m, const T *__restrict__ s, int row, int k0, int end,
+                                              RowPrePair<T> &p)
+{
+    constexpr int STEP = TPR == 1 ? 32 : TPR;
+    row_load<T, TPR>(m, row, k0, end, p.h);
+#pragma unroll
+    for (int j = 0; j < ROW_UNROLL; j++) p.ss[j] = k0 + STEP * j < end ? s[k0 + STEP * j] : (T)0;
+}
+
+template <typename T, int TPR>
+__device__ __forceinline__ void row_prefetch_pair(const MatView<T> &m, const T *__restrict__ s, int row,
+                                                  RowPrePair<T> &p)
+{
+    p.h.k = p.h.end = 0;
+    if (row < m.rows) {
+        lane_range<T, TPR>(m, row, p.h.k, p.h.end);
+        row_load_pair<T, TPR>(m, s, row, p.h.k, p.h.end, p);
+    }
+}
+
+// run chunk() over the row, the first chunk prefetched
+template <typename T, int TPR, typename F>
+__device__ __forceinline__ void row_pair_chunks(const MatView<T> &m, const T *__restrict__ s, int row,
+                                                RowPrePair<T> &p, F chunk)
+{
+    constexpr int STEP = TPR == 1 ? 32 : TPR;
+    if (row >= m.rows) return;
+    const int end = p.h.end;
+    chunk(p.h.k, end);
+    if (m.wmax > ROW_UNROLL)
+        for (int k = p.h.k + STEP * ROW_UNROLL; k < end; k += STEP * ROW_UNROLL) {
+            row_load_pair<T, TPR>(m, s, row, k, end, p);
+            chunk(k, end);
+        }
+}
+
+// sum_j s_rj b_j - (as)_rj x_j; every lane of the group returns it
+template <typename T, int TPR, typename FB, typename FX>
+__device__ __forceinline__ T row_restrict_pair(const MatView<T> &m, const T *__restrict__ s, int row,
+                                               RowPrePair<T> &p, FB bf, FX xf)
+{
+    constexpr int STEP = TPR == 1 ? 32 : TPR;
+    T acc = (T)0;
+    row_pair_chunks<T, TPR>(m, s, row, p, [&](int k0, int end) {
+        T bv[ROW_UNROLL], xv[ROW_UNROLL];
+#pragma unroll
+        for (int j = 0; j < ROW_UNROLL; j++) {
+            const bool ok = k0 + STEP * j < end;
+            bv[j] = ok ? bf(p.h.cc[j]) : (T)0;
+            xv[j] = ok ? xf(p.h.cc[j]) : (T)0;
+        }
+#pragma unroll
+        for (int j = 0; j < ROW_UNROLL; j++)
+            if (k0 + STEP * j < end) acc = rfma(-p.h.vv[j], xv[j], rfma(p.ss[j], bv[j], acc));
+    });
+    if (TPR > 1) {
+#pragma unroll
+        for (int o = TPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, TPR);
+    }
+    return acc;
+}
+
+// ase = sum_j (as)_rj e_j and se = sum_j s_rj e_j; every lane returns both
+template <typename T, int TPR, typename F>
+__device__ __forceinline__ void row_prolong_pair(const MatView<T> &m, const T *__restrict__ s, int row,
+                                                 RowPrePair<T> &p, F ef, T &ase, T &se)
+{
+    constexpr int STEP = TPR == 1 ? 32 : TPR;
+    T a0 = (T)0, a1 = (T)0;
+    row_pair_chunks<T, TPR>(m, s, row, p, [&](int k0, int end) {
+        T ev[ROW_UNROLL];
+#pragma unroll
+        for (int j = 0; j < ROW_UNROLL; j++) ev[j] = k0 + STEP * j < end ? ef(p.h.cc[j]) : (T)0;
+#pragma unroll
+        for (int j = 0; j < ROW_UNROLL; j++)
+            if (k0 + STEP * j < end) {
+                a0 = rfma(p.h.vv[j], ev[j], a0);
+                a1 = rfma(p.ss[j], ev[j], a1);
+            }
+    });
+    if (TPR > 1) {
+#pragma unroll
+        for (int o = TPR / 2; o > 0; o >>= 1) {
+            a0 += __shfl_xor_sync(0xffffffffu, a0, o, TPR);
+            a1 += __shfl_xor_sync(0xffffffffu, a1, o, TPR);
+        }
+    }
+    ase = a0;
+    se = a1;
+}
+
 // a z added to acc, a = ahi + alo (FP32 parts of an FP64 value)
 template <typename Z>
 __device__ __forceinline__ void df_term(DF &acc, float ahi, float alo, Z z);
@@ -259,33 +395,6 @@ __device__ __forceinline__ double row_sum_df(const MatView<float> &m, const floa
 {
     DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, p, z);
     return (double)acc.hi + (double)acc.lo;
-}
-
-// ---- point-wise V-cycle arithmetic with explicit rounding, shared by the
-// level-by-level kernels and the fused coarse cycle so both give the same bits
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-// Chebyshev step at one row: d' = c_d d + c_r D^-1 (b - A x), x' = x + d'
-template <typename T>
-__device__ __forceinline__ void cheb_point(T br, T ax, T ir, T dr, T xr, T cdv, T crv, T &dn, T &xn)
-{
-    T res = rmul(rsub(br, ax), ir);
-    dn = rfma(cdv, dr, rmul(crv, res));
-    xn = radd(xr, dn);
-}
-
-// first step from zero: c D^-1 b
-template <typename T>
-__device__ __forceinline__ T cheb_first_point(T br, T ir, T c)
-{
-    return rmul(c, rmul(br, ir));
 }
 
 // one row of a dense FP32 inverse (rows padded to ld, 16-byte aligned) times
