@@ -175,6 +175,11 @@ struct DevCsr {
     // how the solve phase applies it: tpr = 1 -> SELL-32 below; tpr > 1 -> CSR
     // with tpr lanes per row and the FP32 copy v32
     int tpr = 1;
+    // the CSR of tpr > 1: the canonical arrays, or copies that leave out exact
+    // zeros (x16: column - row as int16, square matrices where every entry fits)
+    int *xp = nullptr, *xi = nullptr;
+    double *xv = nullptr;
+    short *x16 = nullptr;
     float *v32 = nullptr;
     // low FP32 parts, v - (double)(float)v, in the same layout as the solve-phase
     // values (SELL or CSR): with the FP32 values they carry ~48 bits of v
@@ -193,8 +198,8 @@ struct DevCsr {
     // uniform-width SELL only: column - row as int16 when every entry fits
     // (2 instead of 4 bytes of index per stored entry)
     short *sl_ci16 = nullptr;
-    // entries the solve-phase copy holds: the SELL copy leaves out entries
-    // whose value is exactly zero (-1: all nnz entries are held)
+    // entries the solve-phase copy holds: it leaves out entries whose value is
+    // exactly zero (-1: all nnz entries are held)
     int nnz_solve = -1;
 };
 

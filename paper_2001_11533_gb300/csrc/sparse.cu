@@ -325,11 +325,29 @@ __global__ void k_drop_zeros(int rows, const int *__restrict__ rp, const int *__
         }
 }
 
+// column - row of every CSR entry as int16, one thread per row; *bad set if
+// some entry does not fit
+__global__ void k_csr_delta(int rows, const int *__restrict__ rp, const int *__restrict__ ci, short *__restrict__ d16,
+                            int *__restrict__ bad)
+{
+    int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= rows) return;
+    for (int k = rp[r]; k < rp[r + 1]; k++) {
+        int d = ci[k] - r;
+        if (d < -32768 || d > 32767) {
+            atomicOr(bad, 1);
+            d = 0;
+        }
+        d16[k] = (short)d;
+    }
+}
+
 // Solve-phase layout of a.  Entries whose value is exactly zero (the P1
 // stiffness of the Kuhn cube stores 8 of its 15 entries per row as exact
-// zeros) are left out of the SELL copy: a zero term adds nothing to any row
-// sum, so the products are unchanged while the matrix stream shrinks.  The
-// canonical CSR (rp, ci, v) keeps every entry for the setup.
+// zeros, and its Galerkin matrices about half) are left out of the solve-phase
+// copy: a zero term adds nothing to any row sum, so the products are unchanged
+// while the matrix stream shrinks.  The canonical CSR (rp, ci, v) keeps every
+// entry for the setup.
 int prepare_operator(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
 {
     if (a.rows > 0 && a.nnz > 0 && force_tpr <= 1) {
@@ -343,34 +361,26 @@ int prepare_operator(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
         TRY(exclusive_scan<int>(cnt, rp2, a.rows, s, &nz));
         if ((double)nz < 0.95 * a.nnz) {
             DevCsr c = a;
-            c.rp = rp2;
             c.nnz = nz;
-            TRY(sc.alloc(&c.ci, nz));
-            TRY(sc.alloc(&c.v, nz));
+            TRY(ar.alloc(&c.rp, a.rows + 1));
+            TRY(ar.alloc(&c.ci, nz));
+            TRY(ar.alloc(&c.v, nz));
+            CU(cudaMemcpyAsync(c.rp, rp2, sizeof(int) * (a.rows + 1), cudaMemcpyDeviceToDevice, s));
             k_drop_zeros<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.ci, a.v, rp2, c.ci, c.v);
             LAUNCH_CHECK();
-            int longest = 0;
-            TRY(max_row_length(c, s, &longest));
-            const double avg = (double)nz / a.rows;
-            const bool uniform = (double)longest * a.rows <= 1.05 * nz;
-            if (!(avg > 16.0 || (avg > 12.0 && !uniform))) { // SELL-32 for the compacted rows
-                c.tpr = 1;
-                c.wmax = longest;
-                TRY(csr_to_sell(ar, c, 1, s));
-                a.tpr = 1;
-                a.wmax = c.wmax;
-                a.nslices = c.nslices;
-                a.sell_nnz = c.sell_nnz;
-                a.ellw = c.ellw;
-                a.sl_ptr = c.sl_ptr;
-                a.sl_ci = c.sl_ci;
-                a.sl_v = c.sl_v;
-                a.sl_v32 = c.sl_v32;
-                a.sl_ci16 = c.sl_ci16;
-                a.nnz_solve = nz;
-                CU(cudaStreamSynchronize(s));
-                return AMGH_OK;
+            TRY(prepare_layout(ar, c, s, force_tpr));
+            if (c.tpr <= 1) { // SELL-32 has its own copies
+                for (void *q : {(void *)c.rp, (void *)c.ci, (void *)c.v}) ar.release(q);
             }
+            // everything but the canonical CSR
+            c.rp = a.rp;
+            c.ci = a.ci;
+            c.v = a.v;
+            c.nnz = a.nnz;
+            c.longest = 0;
+            c.nnz_solve = nz;
+            a = c;
+            return AMGH_OK;
         }
     }
     return prepare_layout(ar, a, s, force_tpr);
@@ -396,12 +406,29 @@ int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
     // SELL pads every row of a slice to the slice's longest row
     a.wmax = tpr == 1 ? longest : ceil_div(longest, tpr);
     if (tpr == 1) return csr_to_sell(ar, a, 1, s);
+    a.xp = a.rp;
+    a.xi = a.ci;
+    a.xv = a.v;
+    a.x16 = nullptr;
     TRY(ar.alloc(&a.v32, a.nnz));
+    Scratch sc;
+    int *bad = nullptr, hb = 0;
+    short *d16 = nullptr;
     if (a.nnz > 0) {
         k_to_f32<<<ceil_div(a.nnz, 256), 256, 0, s>>>(a.nnz, a.v, a.v32);
         LAUNCH_CHECK();
+        // int16 column offsets where rows and columns number the same things
+        if (a.rows == a.cols) {
+            TRY(sc.alloc(&bad, 1));
+            TRY(ar.alloc(&d16, a.nnz));
+            CU(cudaMemsetAsync(bad, 0, sizeof(int), s));
+            k_csr_delta<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.ci, d16, bad);
+            LAUNCH_CHECK();
+            CU(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+        }
     }
     CU(cudaStreamSynchronize(s));
+    if (d16 && !hb) a.x16 = d16;
     return AMGH_OK;
 }
 
@@ -414,8 +441,8 @@ __global__ void k_lo_parts(int64_t n, const double *__restrict__ v, const float 
 
 int build_lo_parts(Arena &ar, DevCsr &a, cudaStream_t s)
 {
-    int64_t n = a.tpr <= 1 ? a.sell_nnz : a.nnz;
-    const double *v = a.tpr <= 1 ? a.sl_v : a.v;
+    int64_t n = a.tpr <= 1 ? a.sell_nnz : a.nnz_solve >= 0 ? a.nnz_solve : a.nnz;
+    const double *v = a.tpr <= 1 ? a.sl_v : a.xv;
     const float *hi = a.tpr <= 1 ? a.sl_v32 : a.v32;
     TRY(ar.alloc(&a.lo32, n));
     if (n > 0) {
@@ -702,7 +729,7 @@ double spmv_bytes(const DevCsr &a, int vb)
     const double nnz = a.nnz_solve >= 0 ? a.nnz_solve : a.nnz;
     if (a.tpr <= 1 && a.ellw > 0)
         return nnz * (vb + (a.sl_ci16 ? 2 : 4)) + (double)vb * (a.rows + a.cols);
-    return nnz * (vb + 4) + 4.0 * (a.rows + 1) + (double)vb * (a.rows + a.cols);
+    return nnz * (vb + (a.tpr > 1 && a.x16 ? 2 : 4)) + 4.0 * (a.rows + 1) + (double)vb * (a.rows + a.cols);
 }
 
 // ------------------------------------------------------------------ autotuning

@@ -20,7 +20,7 @@ struct MatView {
     const int *ptr; // SELL slice pointers (tpr = 1) or CSR row pointers
     const int *ci;
     const T *v;
-    const short *d16; // SELL: column - row as int16 (DevCsr::sl_ci16), else null
+    const short *d16; // column - row as int16 (DevCsr::sl_ci16, x16), else null
 };
 
 template <typename T>
@@ -29,13 +29,13 @@ template <>
 inline MatView<double> view<double>(const DevCsr &a)
 {
     if (a.tpr <= 1) return {a.rows, a.cols, 1, a.wmax, a.ellw, a.sl_ptr, a.sl_ci, a.sl_v, a.sl_ci16};
-    return {a.rows, a.cols, a.tpr, a.wmax, 0, a.rp, a.ci, a.v, nullptr};
+    return {a.rows, a.cols, a.tpr, a.wmax, 0, a.xp, a.xi, a.xv, a.x16};
 }
 template <>
 inline MatView<float> view<float>(const DevCsr &a)
 {
     if (a.tpr <= 1) return {a.rows, a.cols, 1, a.wmax, a.ellw, a.sl_ptr, a.sl_ci, a.sl_v32, a.sl_ci16};
-    return {a.rows, a.cols, a.tpr, a.wmax, 0, a.rp, a.ci, a.v32, nullptr};
+    return {a.rows, a.cols, a.tpr, a.wmax, 0, a.xp, a.xi, a.v32, a.x16};
 }
 
 // A lane's entries of a row are read ROW_UNROLL at a time: all value and
