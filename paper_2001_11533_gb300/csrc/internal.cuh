@@ -552,6 +552,11 @@ bool mass_cluster_fits(const DevCsr &a, bool df);
 int mass_cluster(amgh_problem *p, const CtrlLevel &C, bool df, const double *b, double *x, CgScal *sc, int cols,
                  double tol, int maxit);
 
+// ------------------------------------------------------------------ state.cu
+// the state CG of level l as one cluster launch, its scalars left in the
+// level's scal; *done = false (and nothing launched) where the level does not fit
+int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol, int maxit, bool *done);
+
 // ------------------------------------------------------------------ assemble.cu
 int assemble_full(amgh_problem *p);
 int extract_sub(Arena &ar, const DevCsr &a, const int *rmap, int nr, const int *cmap, int nc,

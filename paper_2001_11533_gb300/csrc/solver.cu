@@ -522,6 +522,19 @@ int state_solve(amgh_problem *p, int l, const double *f, double *y, double tol, 
     int n = S.A.rows;
     int maxit = p->sopts.inner_max_iter;
     int prec = p->aopts.precision;
+    bool one_launch = false;
+    TRY(state_cluster(p, l, f, y, tol, maxit, &one_launch));
+    if (one_launch) {
+        CgScal h;
+        TRY(read_scal(p, S.scal, &h));
+        // per iteration as the graph-replayed one: V-cycle, product with its dots, update
+        const double mat = prec == 2 ? spmv_bytes(S.A, 4) + 4.0 * S.A.nnz : spmv_bytes(S.A, 8);
+        count_bytes(h.iters * (vcycle_bytes(p, l, prec == 2 ? 4 : 8) + mat + 88.0 * n));
+        p->c_inner_lvl[l] += h.iters;
+        p->c_inner += h.iters;
+        if (iters) *iters = h.iters;
+        return cg_status(h);
+    }
     if (prec != 1) {
         int st = pcg_run(p, l, prec == 2 ? 2 : 0, f, tol, maxit, iters);
         if (prec == 2) TRY(df_to_double(p, n, S.cx, S.scal, y));
