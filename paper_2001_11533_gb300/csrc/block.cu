@@ -1892,7 +1892,7 @@ struct Blk {
         const bool z32 = W.f32 != 0;
         std::function<int()> iter;
         const bool persist = z32 && W.pbar != nullptr;
-        if (!persist && mass_cluster_fits(C.Mu, z32)) { // one cluster per column
+        if (!persist && mass_cluster_fits(C.Mu, z32, maxit)) { // one cluster per column
             TRY(mass_cluster(p, C, z32, b, x, D.mbs->c, K, tol, maxit));
             BScal h;
             TRY(read_bscal(p, D.mbs, &h));

@@ -12,7 +12,10 @@
 
 namespace cg = cooperative_groups;
 
-#define CLUSTER_MAX 16 // CTAs (above 8: not portable, allowed by cluster_allow)
+#define CLUSTER_MAX 16 // CTAs (above 8: not portable, allowed per kernel)
+// a loop that may run longer than this (~0.2 s) is left to the replayed kernels,
+// between which the host reads the stop flag
+#define CLUSTER_MAX_ITERS 10000
 
 __device__ __forceinline__ uint32_t dsmem_of(const void *p, uint32_t rank)
 {

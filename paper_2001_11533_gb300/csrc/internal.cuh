@@ -548,7 +548,7 @@ int prolong_pair(amgh_problem *p, const StateLevel &S, const float *b, const flo
 // whether the mass CG of this level runs as one cluster launch; the launch:
 // cols right sides interleaved (element i of column c at i * cols + c), the
 // final scalars of column c in sc[c]
-bool mass_cluster_fits(const DevCsr &a, bool df);
+bool mass_cluster_fits(const DevCsr &a, bool df, int maxit);
 int mass_cluster(amgh_problem *p, const CtrlLevel &C, bool df, const double *b, double *x, CgScal *sc, int cols,
                  double tol, int maxit);
 

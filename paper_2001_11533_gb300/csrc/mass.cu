@@ -238,10 +238,10 @@ static int mass_dispatch(amgh_problem *p, const MassShape &sh, const DevCsr &a, 
     }
 }
 
-bool mass_cluster_fits(const DevCsr &a, bool df)
+bool mass_cluster_fits(const DevCsr &a, bool df, int maxit)
 {
     MassShape sh;
-    return mass_shape(a, df, &sh);
+    return maxit <= CLUSTER_MAX_ITERS && mass_shape(a, df, &sh);
 }
 
 int mass_cluster(amgh_problem *p, const CtrlLevel &C, bool df, const double *b, double *x, CgScal *sc, int cols,

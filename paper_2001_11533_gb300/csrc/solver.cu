@@ -574,7 +574,7 @@ int mass_solve(amgh_problem *p, int l, const double *b, double *x, int64_t *iter
     int n = C.Mu.rows;
     // precision 2: the mass CG in double-float too, Jacobi from FP32 copies
     bool df = p->aopts.precision == 2;
-    if (mass_cluster_fits(C.Mu, df)) {
+    if (mass_cluster_fits(C.Mu, df, p->sopts.mass_max_iter)) {
         timer_begin(p, KC_VEC);
         TRY(mass_cluster(p, C, df, b, x, C.mscal, 1, p->sopts.mass_tol, p->sopts.mass_max_iter));
         timer_end(p, KC_VEC, 48.0 * n);

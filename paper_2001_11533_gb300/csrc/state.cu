@@ -451,7 +451,7 @@ int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol
 {
     *done = true;
     size_t smem = 0;
-    if (p->aopts.precision == 2) {
+    if (p->aopts.precision == 2 && maxit <= CLUSTER_MAX_ITERS) {
         ScgArgs<float> a = {};
         if (scg_shape<float>(p, l, &a, &smem)) {
             for (int k = 0; k < a.levels; k++) a.lv[k].invd = p->sl[l + k].invd32;
@@ -459,7 +459,7 @@ int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol
             a.ld = p->Acoarse.ld32;
             return scg_launch<ClusterDf>(p, l, a, smem, f, y, tol, maxit);
         }
-    } else if (p->aopts.precision == 0) {
+    } else if (p->aopts.precision == 0 && maxit <= CLUSTER_MAX_ITERS) {
         ScgArgs<double> a = {};
         if (scg_shape<double>(p, l, &a, &smem)) {
             for (int k = 0; k < a.levels; k++) a.lv[k].invd = p->sl[l + k].invd;

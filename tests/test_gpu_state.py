@@ -81,3 +81,20 @@ def test_statuses(N, precision):
         p.state_solve_level(0, cuda(b), TOL)
     assert e.value.code == -7
     p.close()
+
+
+# a cap above which the loop is replayed (csrc/clustercg.cuh) instead: same answer
+@pytest.mark.parametrize("cap", [10000, 10001])
+@pytest.mark.parametrize("precision", [0, 2])
+def test_iteration_caps(precision, cap):
+    p = problem("square", 33, precision)
+    p.set_solve_opts(inner_max_iter=cap, mass_max_iter=cap, mass_tol=TOL)
+    for which, solve, n in (("A", lambda b: p.state_solve_level(0, b, TOL), p.sizes["m"]),
+                            ("Mu", lambda b: p.mass_solve(0, b), p.sizes["n"])):
+        rp, ci, v, shape = p.matrix(which, 0)
+        A = sp.csr_matrix((v, ci, rp), shape=shape)
+        b = np.random.default_rng(5).standard_normal(n)
+        x, it = solve(cuda(b))
+        assert 0 < it <= 100
+        assert np.linalg.norm(A @ x.cpu().numpy() - b) <= 2 * TOL * np.linalg.norm(b)
+    p.close()
