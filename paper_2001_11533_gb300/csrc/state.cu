@@ -10,7 +10,7 @@
 //
 //   rows      level k's rows are dealt in runs of 2^lg_k to the CTAs, so the owner
 //             of a column is a shift; as many lanes share a row as the CTA has
-//             threads for, so a lane has one to a few entries
+//             threads for, so a lane has two to a few entries
 //   matrices  of every level in the owner's shared memory, copied once per solve,
 //             columns as the addresses of their vector elements.  (Read from L2
 //             in each phase, rows loaded ahead of the barrier, the solves were
@@ -27,20 +27,24 @@
 // lanes of a row, which depend on the hierarchy only.  The stopping test comes
 // beside the next scalar step, as in mass.cu.
 //
-// What bounds it: dependent latency, about 1,600 cycles a phase (barrier, record
-// of the phase, gather, sum over the row's lanes, point-wise step) and 5,000 for
-// the sums and the scalar step.  Measured (one GB300, whole public call to 1e-10,
-// 16-19 iterations, graph-replayed -> here, us): FP32 V-cycles 49 rows 339 -> 182,
-// 441 rows 468 -> 319, 961 rows 379 -> 240, 2,025 rows 541 -> 356 (FP64: 461 ->
-// 345, 709 -> 566, 524 -> 421, 771 -> 640).  Rows per CTA from 32 to 128 make no
-// difference beyond 5 %.
+// What bounds it: dependent latency and issue.  A phase is about 1,400 cycles (a
+// cluster barrier 600, the gather 300, the sum over a row's lanes, the point-wise
+// step), the sums and the scalar step of an iteration 5,000.  Measured (one GB300,
+// whole public call to 1e-10, 16-19 iterations, us, graph-replayed -> here): FP32
+// V-cycles 49 rows 339 -> 169, 441 rows 468 -> 292, 961 rows 379 -> 229, 2,025 rows
+// 541 -> 332; FP64 461 -> 243, 709 -> 390, 524 -> 307, 771 -> 452.  Rows per CTA
+// from 32 to 128 make no difference beyond 5 %.
 #include <algorithm>
 #include <atomic>
 
 #include "clustercg.cuh"
 #include "spmv.cuh"
 
-#define SCG_TPB 512
+// With 512 threads and a lane per entry the warps spent their issue slots (39 %
+// busy) on phase bookkeeping and on butterflies over nearly empty lanes, in FP64
+// one addition of a whole warp a step: 2,025 rows 358 us, FP64 665; with 256
+// threads, at least two entries a lane and idle warps skipping the phase 332, 452.
+#define SCG_TPB 256
 #define SCG_ROWS 128 // rows of the solved level per CTA
 #define SCG_LEVELS 6
 #define SCG_SMEM (200 << 10)
@@ -160,6 +164,10 @@ __device__ __forceinline__ typename ScgSum<M, PROD>::V scg_row(const ScgCta<type
         }
     };
     scg_arrive(c.ctas);
+    if (t >= m.width) { // a warp without entries (the width is a multiple of 32)
+        scg_wait(c.ctas);
+        return Sum::zero();
+    }
     load(0);
     scg_wait(c.ctas);
     typename Sum::V s = Sum::zero();
@@ -343,12 +351,12 @@ __global__ void __launch_bounds__(SCG_TPB, 1)
 
 // ------------------------------------------------------------------ host side
 // Place m's rows (dealt in runs of 2^lg) in shared memory: as many lanes a row
-// as the threads allow and its longest row fills.
+// as the threads allow and its longest row fills with two entries each.
 static bool scg_place(const DevCsr &a, int lg, size_t vb, bool pair, ScgMat *m, int64_t *off)
 {
     if (a.rows < 1 || a.longest < 1) return false;
     int lgl = 0;
-    while (lgl < 5 && (2 << lgl << lg) <= SCG_TPB && (1 << lgl) < a.longest) lgl++;
+    while (lgl < 5 && (2 << lgl << lg) <= SCG_TPB && (2 << lgl) < a.longest) lgl++;
     const int width = std::max(32, 1 << lg << lgl), entries = ceil_div(a.longest, 1 << lgl);
     if (width > SCG_TPB || entries > SCG_MAX_ENTRIES) return false;
     const int64_t each = (int64_t)entries * width;
