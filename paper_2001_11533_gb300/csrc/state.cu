@@ -10,7 +10,7 @@
 //
 //   rows      level k's rows are dealt in runs of 2^lg_k to the CTAs, so the owner
 //             of a column is a shift; as many lanes share a row as the CTA has
-//             threads for, so a lane has two to a few entries
+//             threads for, so a lane has one or two to a few entries
 //   matrices  of every level in the owner's shared memory, copied once per solve,
 //             columns as the addresses of their vector elements.  (Read from L2
 //             in each phase, rows loaded ahead of the barrier, the solves were
@@ -31,8 +31,8 @@
 // cluster barrier 600, the gather 300, the sum over a row's lanes, the point-wise
 // step), the sums and the scalar step of an iteration 5,000.  Measured (one GB300,
 // whole public call to 1e-10, 16-19 iterations, us, graph-replayed -> here): FP32
-// V-cycles 49 rows 339 -> 169, 441 rows 468 -> 292, 961 rows 379 -> 229, 2,025 rows
-// 541 -> 332; FP64 461 -> 243, 709 -> 390, 524 -> 307, 771 -> 452.  Rows per CTA
+// V-cycles 49 rows 339 -> 182, 441 rows 468 -> 319, 961 rows 379 -> 240, 2,025 rows
+// 541 -> 356; FP64 461 -> 243, 709 -> 390, 524 -> 307, 771 -> 452.  Rows per CTA
 // from 32 to 128 make no difference beyond 5 %.
 #include <algorithm>
 #include <atomic>
@@ -40,11 +40,14 @@
 #include "clustercg.cuh"
 #include "spmv.cuh"
 
-// With 512 threads and a lane per entry the warps spent their issue slots (39 %
-// busy) on phase bookkeeping and on butterflies over nearly empty lanes, in FP64
-// one addition of a whole warp a step: 2,025 rows 358 us, FP64 665; with 256
-// threads, at least two entries a lane and idle warps skipping the phase 332, 452.
-#define SCG_TPB 256
+// Threads of a CTA.  FP64: with 512 and a lane per entry the FP64 units are held
+// by butterflies over nearly empty lanes, one addition of a whole warp a step;
+// with 256, at least two entries a lane and idle warps skipping the phase 2,025
+// rows take 452 us instead of 665 (33^2 cost and gradient 1.40 -> 1.12 ms).  FP32
+// solves alone gain 7 % by the same, but whole calls lose 1 % (65^2 solve 13.43 ->
+// 13.55 ms, 201^2 preconditioner 4.51 -> 4.56), so they keep the wider form.
+template <typename T>
+constexpr int SCG_TPB = sizeof(T) == 8 ? 256 : 512;
 #define SCG_ROWS 128 // rows of the solved level per CTA
 #define SCG_LEVELS 6
 #define SCG_SMEM (200 << 10)
@@ -164,7 +167,7 @@ __device__ __forceinline__ typename ScgSum<M, PROD>::V scg_row(const ScgCta<type
         }
     };
     scg_arrive(c.ctas);
-    if (t >= m.width) { // a warp without entries (the width is a multiple of 32)
+    if (sizeof(T) == 8 && t >= m.width) { // a warp without entries (the width is a multiple of 32)
         scg_wait(c.ctas);
         return Sum::zero();
     }
@@ -201,10 +204,10 @@ __device__ __forceinline__ void scg_dense(const ScgCta<T> &c, const ScgArgs<T> &
     const T *b = c.vec(L, SV_B), *inv = (const T *)(c.sm + a.inv_off);
     T *all = (T *)(c.sm + a.b_off), *x = c.vec(L, SV_XB);
     cluster_barrier(c.ctas);
-    for (int j = t; j < n; j += SCG_TPB)
+    for (int j = t; j < n; j += SCG_TPB<T>)
         all[j] = dsmem_ld(dsmem_of(b + (j & ((1 << L.lg) - 1)), (uint32_t)(j >> L.lg)), T());
     __syncthreads();
-    for (int i = t >> 5; i < mine; i += SCG_TPB / 32) {
+    for (int i = t >> 5; i < mine; i += SCG_TPB<T> / 32) {
         T s0 = 0, s1 = 0;
         int j = t & 31;
         for (; j + 32 < n; j += 64) {
@@ -277,7 +280,7 @@ __device__ __forceinline__ float scg_head(DF r) { return r.hi; }
 __device__ __forceinline__ double scg_head(double r) { return r; }
 
 template <typename M>
-__global__ void __launch_bounds__(SCG_TPB, 1)
+__global__ void __launch_bounds__(SCG_TPB<typename M::Z>, 1)
     k_state_cg(const __grid_constant__ ScgArgs<typename M::Z> a, const double *__restrict__ f, double *__restrict__ y,
                CgScal *scal, double tol2, int maxit)
 {
@@ -305,7 +308,7 @@ __global__ void __launch_bounds__(SCG_TPB, 1)
         const ScgLevel &L = a.lv[a.levels - 1];
         const int first = (int)c.rank << L.lg, mine = min(1 << L.lg, L.n - first);
         T *inv = (T *)(c.sm + a.inv_off);
-        for (int i = t >> 5; i < mine; i += SCG_TPB / 32)
+        for (int i = t >> 5; i < mine; i += SCG_TPB<T> / 32)
             for (int j = t & 31; j < L.n; j += 32) inv[i * L.n + j] = a.inv[(int64_t)(first + i) * a.ld + j];
     }
     const ScgLevel &L = a.lv[0];
@@ -351,14 +354,15 @@ __global__ void __launch_bounds__(SCG_TPB, 1)
 
 // ------------------------------------------------------------------ host side
 // Place m's rows (dealt in runs of 2^lg) in shared memory: as many lanes a row
-// as the threads allow and its longest row fills with two entries each.
+// as the threads allow and its longest row fills (FP64: with two entries each).
 static bool scg_place(const DevCsr &a, int lg, size_t vb, bool pair, ScgMat *m, int64_t *off)
 {
     if (a.rows < 1 || a.longest < 1) return false;
+    const int tpb = vb == 8 ? SCG_TPB<double> : SCG_TPB<float>, least = vb == 8 ? 2 : 1; // entries a lane
     int lgl = 0;
-    while (lgl < 5 && (2 << lgl << lg) <= SCG_TPB && (2 << lgl) < a.longest) lgl++;
+    while (lgl < 5 && (2 << lgl << lg) <= tpb && (least << lgl) < a.longest) lgl++;
     const int width = std::max(32, 1 << lg << lgl), entries = ceil_div(a.longest, 1 << lgl);
-    if (width > SCG_TPB || entries > SCG_MAX_ENTRIES) return false;
+    if (width > tpb || entries > SCG_MAX_ENTRIES) return false;
     const int64_t each = (int64_t)entries * width;
     *m = ScgMat{a.rp, a.ci, a.v, a.rows, lg, lgl, entries, width, (int)*off, -1, 0};
     *off += each * vb;
@@ -443,7 +447,7 @@ static int scg_launch(amgh_problem *p, int l, ScgArgs<typename M::Z> &a, size_t 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(a.ctas, 1, 1);
-    cfg.blockDim = dim3(SCG_TPB, 1, 1);
+    cfg.blockDim = dim3(SCG_TPB<typename M::Z>, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = p->stream;
     cfg.attrs = attr;
