@@ -746,8 +746,10 @@ extern "C" int amgh_mass_solve(amgh_problem *p, int level, const double *b, doub
     NEED_SETUP(p);
     CallScope cs_(p);
     if (level < 0 || level >= p->Lc || !b || !x) return AMGH_ERR_INVALID_ARG;
-    TRY(mass_solve(p, level, b, x, iters));
-    return sync_stream(p);
+    int st = mass_solve(p, level, b, x, iters);
+    if (p->pm_bar) return finish_call(p, st); // the persistent form's barriers may have given up
+    int s2 = sync_stream(p);
+    return st != AMGH_OK ? st : s2;
 }
 
 extern "C" int amgh_hessian_apply_level(amgh_problem *p, int level, const double *v, double *hv)

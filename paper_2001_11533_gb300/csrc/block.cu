@@ -2484,5 +2484,5 @@ int persistent_mass_single(amgh_problem *p, int l, const double *b, double *x, i
     p->c_mass_lvl[l] += h.iters;
     p->c_mass += h.iters;
     if (iters) *iters = h.iters;
-    return AMGH_OK;
+    return col_status(h);
 }
