@@ -263,6 +263,7 @@ static void reset_hierarchy(amgh_problem *p)
     block_free(p);
     solver_free_graphs(p);
     p->harena.free_all();
+    p->pm_bs = p->pm_p1 = p->pm_p2 = p->pm_bar = nullptr; // they lay in the arena
     for (int l = 0; l < AMGH_MAXL; l++) {
         p->sl[l] = StateLevel();
         p->cl[l] = CtrlLevel();

@@ -96,3 +96,18 @@ def test_batch_keeps_cooperative_launches_off_on_large_levels():
         out.append(([x.cpu().numpy() for x in u], amgh.launch_count() - n0))
     assert all(np.array_equal(a, b) for a, b in zip(out[0][0], out[1][0]))
     assert out[0][1] == out[1][1]
+
+
+def test_second_setup_makes_new_work_space():
+    """The work space of the persistent solves goes with the hierarchy that it
+    was allocated beside: a second setup on the handle starts without it."""
+    p, fresh = problem(129, persistent_cg=1), problem(129, persistent_cg=1)
+    b = cuda(np.random.default_rng(2).standard_normal(p.sizes["n"]))
+    p.mass_solve(0, b)
+    p.amg_setup(precision=2, coarse_max=64, persistent_cg=1)
+    p.amg_setup(precision=2, coarse_max=256, persistent_cg=1)
+    x, it = p.mass_solve(0, b)
+    y, it0 = fresh.mass_solve(0, b)
+    assert it == it0 and np.array_equal(x.cpu().numpy(), y.cpu().numpy())
+    p.close()
+    fresh.close()
