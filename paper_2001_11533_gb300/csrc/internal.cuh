@@ -188,7 +188,7 @@ struct DevCsr {
     // the widest slice; CSR: ceil(longest row / tpr)); rows up to
     // ROW_UNROLL per lane are read with every load issued up front
     int wmax = 1 << 30;
-    int longest = 0; // entries of the longest CSR row (0: not known)
+    int longest = 0; // entries of the longest canonical CSR row, exact zeros included (0: no layout yet)
     // SELL-32; ellw > 0: every slice has this width (slice s starts at
     // 32 * ellw * s, so kernels need not load the slice pointers)
     int nslices = 0, sell_nnz = 0, ellw = 0;

@@ -377,7 +377,7 @@ int prepare_operator(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
             c.ci = a.ci;
             c.v = a.v;
             c.nnz = a.nnz;
-            c.longest = 0;
+            TRY(max_row_length(a, s, &c.longest));
             c.nnz_solve = nz;
             a = c;
             return AMGH_OK;
