@@ -569,6 +569,12 @@ int amgh_fp64_peak(int kind, void *stream, double *tflops);
  * of about 64 ns).  Process-wide.  Errors: INVALID_ARG below -1, CUDA. */
 int amgh_debug_grid_polls(int polls);
 
+/* Test hook: clusters of more than `ctas` CTAs count as ones that the device
+ * cannot place, so that the one-launch CG solves of small levels take the
+ * replayed kernels as they do on such a device; -1 restores the default (the
+ * device is asked).  Process-wide.  Errors: INVALID_ARG below -1. */
+int amgh_debug_cluster_ctas(int ctas);
+
 /* Number of kernels this library launched since load (all problems). */
 int64_t amgh_launch_count(void);
 

@@ -102,6 +102,7 @@ _SIGS = {
     "amgh_dense_spd_inverse": ([_I, _P, _P, _P, _P], _I),
     "amgh_fp64_peak": ([_I, _P, _P], _I),
     "amgh_debug_grid_polls": ([_I], _I),
+    "amgh_debug_cluster_ctas": ([_I], _I),
     "amgh_batch_create": ([_P, _I, _P], _I),
     "amgh_batch_setup": ([_P, _P], _I),
     "amgh_batch_set_workers": ([_P, _I], _I),
@@ -204,6 +205,12 @@ def debug_grid_polls(polls: int = -1):
     """amgh_debug_grid_polls: poll limit of every software grid barrier wait
     (-1 = default); a test hook for the timeout path."""
     check(lib().amgh_debug_grid_polls(int(polls)), "amgh_debug_grid_polls")
+
+
+def debug_cluster_ctas(ctas: int = -1):
+    """amgh_debug_cluster_ctas: the largest cluster that counts as placeable
+    (-1 = ask the device); a test hook for the fallback of the one-launch solves."""
+    check(lib().amgh_debug_cluster_ctas(int(ctas)), "amgh_debug_cluster_ctas")
 
 
 def fp64_peak(kind: int, stream=None) -> float:

@@ -906,6 +906,13 @@ extern "C" int amgh_debug_limits(int bulk_first_polls, int mis_round_cap, int pr
     return bulk_set_first_polls(bulk_first_polls);
 }
 
+extern "C" int amgh_debug_cluster_ctas(int ctas)
+{
+    if (ctas < -1) return AMGH_ERR_INVALID_ARG;
+    cluster_set_ctas(ctas);
+    return AMGH_OK;
+}
+
 extern "C" int amgh_debug_grid_polls(int polls)
 {
     if (polls < -1) return AMGH_ERR_INVALID_ARG;

@@ -1892,8 +1892,9 @@ struct Blk {
         const bool z32 = W.f32 != 0;
         std::function<int()> iter;
         const bool persist = z32 && W.pbar != nullptr;
-        if (!persist && mass_cluster_fits(C.Mu, z32, maxit)) { // one cluster per column
-            TRY(mass_cluster(p, C, z32, b, x, D.mbs->c, K, tol, maxit));
+        bool one_launch = false; // one cluster per column
+        if (!persist) TRY(mass_cluster(p, C, z32, b, x, D.mbs->c, K, tol, maxit, &one_launch));
+        if (one_launch) {
             BScal h;
             TRY(read_bscal(p, D.mbs, &h));
             for (int c = 0; c < K; c++) {

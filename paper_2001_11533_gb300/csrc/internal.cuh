@@ -39,6 +39,12 @@ void amgh_note_msg(const char *msg);
 void amgh_count_launch(int n = 1);
 // blocks of `block` threads of `kernel` resident on the current device at once
 int resident_grid(const void *kernel, int block);
+// whether the current device can place a cluster of `ctas` CTAs of `kernel` (of
+// at most smem_max bytes of dynamic shared memory), which a partitioned or
+// narrower one may not; asked once per kernel, device and shape, and left
+// allowed for the launch
+bool cluster_fits(const void *kernel, int ctas, int threads, size_t smem, size_t smem_max);
+void cluster_set_ctas(int ctas);
 void amgh_set_capturing(int on);
 // Programmatic dependent launch.  Solve-phase kernels are launched with
 // pdl_launch, which lets a kernel be scheduled while its predecessor in the
@@ -545,16 +551,17 @@ int prolong_pair(amgh_problem *p, const StateLevel &S, const float *b, const flo
                  float *xn, double c, const int *skip);
 
 // ------------------------------------------------------------------ mass.cu
-// whether the mass CG of this level runs as one cluster launch; the launch:
-// cols right sides interleaved (element i of column c at i * cols + c), the
-// final scalars of column c in sc[c]
-bool mass_cluster_fits(const DevCsr &a, bool df, int maxit);
+// the mass CG of a level as one cluster launch: cols right sides interleaved
+// (element i of column c at i * cols + c), the final scalars of column c in
+// sc[c]; *done = false (and nothing launched) where the level does not fit or
+// the device cannot place the cluster
 int mass_cluster(amgh_problem *p, const CtrlLevel &C, bool df, const double *b, double *x, CgScal *sc, int cols,
-                 double tol, int maxit);
+                 double tol, int maxit, bool *done);
 
 // ------------------------------------------------------------------ state.cu
 // the state CG of level l as one cluster launch, its scalars left in the
 // level's scal; *done = false (and nothing launched) where the level does not fit
+// or the device cannot place the cluster
 int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol, int maxit, bool *done);
 
 // ------------------------------------------------------------------ assemble.cu

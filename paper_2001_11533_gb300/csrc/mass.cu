@@ -40,7 +40,6 @@
 // 2,278 rows 421 -> 137, 4,225 rows 384 -> 123 (FP64: 339 -> 86, 459 -> 123,
 // 486 -> 198, 439 -> 180).
 #include <algorithm>
-#include <atomic>
 
 #include "internal.cuh"
 #include "clustercg.cuh"
@@ -185,18 +184,11 @@ static bool mass_shape(const DevCsr &a, bool df, MassShape *out)
 
 template <typename M, int L, int E>
 static int mass_launch_as(amgh_problem *p, const MassShape &sh, const DevCsr &a, const void *invd,
-                          const MassRhs &rhs, double tol, int maxit)
+                          const MassRhs &rhs, double tol, int maxit, bool *done)
 {
     auto kern = k_mass_cg<M, L, E>;
-    // clusters above 8 CTAs: allowed once per instantiation and device
-    static std::atomic<uint64_t> allowed{0};
-    int dev = 0;
-    CU(cudaGetDevice(&dev));
-    const uint64_t bit = 1ull << (dev & 63);
-    if (!(allowed.load() & bit)) {
-        CU(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        allowed.fetch_or(bit);
-    }
+    *done = cluster_fits((const void *)kern, sh.ctas, sh.threads, 0, 0);
+    if (!*done) return AMGH_OK;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -218,38 +210,33 @@ static int mass_launch_as(amgh_problem *p, const MassShape &sh, const DevCsr &a,
 
 template <typename M, int L>
 static int mass_launch(amgh_problem *p, const MassShape &sh, const DevCsr &a, const void *invd, const MassRhs &rhs,
-                       double tol, int maxit)
+                       double tol, int maxit, bool *done)
 {
-    if (sh.entries == 8) return mass_launch_as<M, L, 8>(p, sh, a, invd, rhs, tol, maxit);
-    return mass_launch_as<M, L, 16>(p, sh, a, invd, rhs, tol, maxit);
+    if (sh.entries == 8) return mass_launch_as<M, L, 8>(p, sh, a, invd, rhs, tol, maxit, done);
+    return mass_launch_as<M, L, 16>(p, sh, a, invd, rhs, tol, maxit, done);
 }
 
 template <typename M>
 static int mass_dispatch(amgh_problem *p, const MassShape &sh, const DevCsr &a, const void *invd, const MassRhs &rhs,
-                         double tol, int maxit)
+                         double tol, int maxit, bool *done)
 {
     switch (sh.lanes) {
-    case 2: return mass_launch<M, 2>(p, sh, a, invd, rhs, tol, maxit);
-    case 4: return mass_launch<M, 4>(p, sh, a, invd, rhs, tol, maxit);
-    case 8: return mass_launch<M, 8>(p, sh, a, invd, rhs, tol, maxit);
-    case 16: return mass_launch<M, 16>(p, sh, a, invd, rhs, tol, maxit);
-    case 32: return mass_launch<M, 32>(p, sh, a, invd, rhs, tol, maxit);
-    default: return mass_launch<M, 1>(p, sh, a, invd, rhs, tol, maxit);
+    case 2: return mass_launch<M, 2>(p, sh, a, invd, rhs, tol, maxit, done);
+    case 4: return mass_launch<M, 4>(p, sh, a, invd, rhs, tol, maxit, done);
+    case 8: return mass_launch<M, 8>(p, sh, a, invd, rhs, tol, maxit, done);
+    case 16: return mass_launch<M, 16>(p, sh, a, invd, rhs, tol, maxit, done);
+    case 32: return mass_launch<M, 32>(p, sh, a, invd, rhs, tol, maxit, done);
+    default: return mass_launch<M, 1>(p, sh, a, invd, rhs, tol, maxit, done);
     }
 }
 
-bool mass_cluster_fits(const DevCsr &a, bool df, int maxit)
-{
-    MassShape sh;
-    return maxit <= CLUSTER_MAX_ITERS && mass_shape(a, df, &sh);
-}
-
 int mass_cluster(amgh_problem *p, const CtrlLevel &C, bool df, const double *b, double *x, CgScal *sc, int cols,
-                 double tol, int maxit)
+                 double tol, int maxit, bool *done)
 {
     MassShape sh;
-    if (!mass_shape(C.Mu, df, &sh)) return AMGH_ERR_INVALID_ARG;
+    *done = false;
+    if (maxit > CLUSTER_MAX_ITERS || !mass_shape(C.Mu, df, &sh)) return AMGH_OK;
     const MassRhs rhs = {b, x, sc, cols};
-    return df ? mass_dispatch<ClusterDf>(p, sh, C.Mu, C.mu_invdiag32, rhs, tol, maxit)
-              : mass_dispatch<ClusterF64>(p, sh, C.Mu, C.mu_invdiag, rhs, tol, maxit);
+    return df ? mass_dispatch<ClusterDf>(p, sh, C.Mu, C.mu_invdiag32, rhs, tol, maxit, done)
+              : mass_dispatch<ClusterF64>(p, sh, C.Mu, C.mu_invdiag, rhs, tol, maxit, done);
 }

@@ -574,9 +574,11 @@ int mass_solve(amgh_problem *p, int l, const double *b, double *x, int64_t *iter
     int n = C.Mu.rows;
     // precision 2: the mass CG in double-float too, Jacobi from FP32 copies
     bool df = p->aopts.precision == 2;
-    if (mass_cluster_fits(C.Mu, df, p->sopts.mass_max_iter)) {
-        timer_begin(p, KC_VEC);
-        TRY(mass_cluster(p, C, df, b, x, C.mscal, 1, p->sopts.mass_tol, p->sopts.mass_max_iter));
+    bool one_launch = false;
+    const size_t mark = p->timer.ev.size();
+    timer_begin(p, KC_VEC);
+    TRY(mass_cluster(p, C, df, b, x, C.mscal, 1, p->sopts.mass_tol, p->sopts.mass_max_iter, &one_launch));
+    if (one_launch) {
         timer_end(p, KC_VEC, 48.0 * n);
         CgScal h;
         TRY(read_scal(p, C.mscal, &h));
@@ -588,6 +590,7 @@ int mass_solve(amgh_problem *p, int l, const double *b, double *x, int64_t *iter
         if (iters) *iters = h.iters;
         return cg_status(h);
     }
+    timer_drop_from(p, mark);
     if (df && p->aopts.persistent_cg && !p->parent && !p->in_batch && !p->capturing)
         return persistent_mass_single(p, l, b, x, iters);
     if (df) {

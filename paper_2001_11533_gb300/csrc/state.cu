@@ -35,7 +35,6 @@
 // 541 -> 356; FP64 461 -> 243, 709 -> 390, 524 -> 307, 771 -> 452.  Rows per CTA
 // from 32 to 128 make no difference beyond 5 %.
 #include <algorithm>
-#include <atomic>
 
 #include "clustercg.cuh"
 #include "spmv.cuh"
@@ -432,18 +431,11 @@ static bool scg_shape(const amgh_problem *p, int l, ScgArgs<T> *a, size_t *smem)
 
 template <typename M>
 static int scg_launch(amgh_problem *p, int l, ScgArgs<typename M::Z> &a, size_t smem, const double *f, double *y,
-                      double tol, int maxit)
+                      double tol, int maxit, bool *done)
 {
     auto kern = k_state_cg<M>;
-    static std::atomic<uint64_t> allowed{0}; // attributes set, per device
-    int dev = 0;
-    CU(cudaGetDevice(&dev));
-    const uint64_t bit = 1ull << (dev & 63);
-    if (!(allowed.load() & bit)) {
-        CU(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SCG_SMEM));
-        allowed.fetch_or(bit);
-    }
+    *done = cluster_fits((const void *)kern, a.ctas, SCG_TPB<typename M::Z>, smem, SCG_SMEM);
+    if (!*done) return AMGH_OK;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -465,9 +457,10 @@ static int scg_launch(amgh_problem *p, int l, ScgArgs<typename M::Z> &a, size_t 
 
 // The state CG of level l as one cluster launch, its scalars left in the
 // level's scal; *done = false (and nothing launched) where the level does not fit
+// or the device cannot place the cluster
 int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol, int maxit, bool *done)
 {
-    *done = true;
+    *done = false;
     size_t smem = 0;
     if (p->aopts.precision == 2 && maxit <= CLUSTER_MAX_ITERS) {
         ScgArgs<float> a = {};
@@ -475,7 +468,7 @@ int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol
             for (int k = 0; k < a.levels; k++) a.lv[k].invd = p->sl[l + k].invd32;
             a.inv = p->Acoarse.inv32;
             a.ld = p->Acoarse.ld32;
-            return scg_launch<ClusterDf>(p, l, a, smem, f, y, tol, maxit);
+            return scg_launch<ClusterDf>(p, l, a, smem, f, y, tol, maxit, done);
         }
     } else if (p->aopts.precision == 0 && maxit <= CLUSTER_MAX_ITERS) {
         ScgArgs<double> a = {};
@@ -483,9 +476,8 @@ int state_cluster(amgh_problem *p, int l, const double *f, double *y, double tol
             for (int k = 0; k < a.levels; k++) a.lv[k].invd = p->sl[l + k].invd;
             a.inv = p->Acoarse.inv;
             a.ld = p->Acoarse.n;
-            return scg_launch<ClusterF64>(p, l, a, smem, f, y, tol, maxit);
+            return scg_launch<ClusterF64>(p, l, a, smem, f, y, tol, maxit, done);
         }
     }
-    *done = false;
     return AMGH_OK;
 }

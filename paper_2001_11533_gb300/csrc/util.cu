@@ -4,7 +4,9 @@
 #include <string.h>
 
 #include <atomic>
+#include <map>
 #include <mutex>
+#include <tuple>
 
 #include "internal.cuh"
 #include "util.cuh"
@@ -67,6 +69,50 @@ int resident_grid(const void *kernel, int block)
     cache.push_back({{kernel, dev}, g});
     return g;
 }
+
+// largest cluster that counts as placeable; lowered only by amgh_debug_cluster_ctas
+static std::atomic<int> g_cluster_ctas{1 << 30};
+void cluster_set_ctas(int ctas) { g_cluster_ctas = ctas < 0 ? 1 << 30 : ctas; }
+
+bool cluster_fits(const void *kernel, int ctas, int threads, size_t smem, size_t smem_max)
+{
+    typedef std::tuple<const void *, int, int, int, size_t> Key;
+    static std::mutex mu;
+    static std::map<Key, bool> cache;
+    if (ctas > g_cluster_ctas.load()) return false;
+    smem = (smem + 8191) / 8192 * 8192; // asked in steps of 8 KB
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    const Key key(kernel, dev, ctas, threads, smem);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    bool ok = smem <= smem_max;
+    // clusters above 8 CTAs and more than 48 KB are allowed per kernel and device
+    if (ok && ctas > 8)
+        ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (ok && smem_max > 0)
+        ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max) == cudaSuccess;
+    if (ok) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ctas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(ctas, 1, 1);
+        cfg.blockDim = dim3(threads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        ok = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+    }
+    if (!ok) cudaGetLastError();
+    cache[key] = ok;
+    return ok;
+}
+
 extern "C" int64_t amgh_launch_count(void) { return (int64_t)g_launches.load(); }
 
 // ------------------------------------------------------------------ memory pool

@@ -61,3 +61,52 @@ def test_first_level_past_the_cluster_is_replayed(precision):
     p.state_solve_level(0, torch.ones(n, dtype=torch.float64, device="cuda"), TOL)
     assert amgh.launch_count() - n0 > 1
     p.close()
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_falls_back_where_no_cluster_can_be_placed(precision):
+    """A device that cannot place the clusters (here: none above one CTA counts)
+    answers the same calls by the replayed kernels."""
+    import torch
+    from paper_2001_11533_gb300 import amgh
+    p = problem("jittered", 33, precision, 16)
+    p.set_solve_opts(mass_tol=TOL)
+    rng = np.random.default_rng(33)
+    for which, solve, n in (("A", lambda b: p.state_solve_level(0, b, TOL), p.sizes["m"]),
+                            ("Mu", lambda b: p.mass_solve(0, b), p.sizes["n"])):
+        rp, ci, v, shape = p.matrix(which, 0)
+        A = sp.csr_matrix((v, ci, rp), shape=shape)
+        f = rng.standard_normal(n)
+        counts, iters = [], []
+        try:
+            for ctas in (-1, 1, -1):
+                amgh.debug_cluster_ctas(ctas)
+                n0 = amgh.launch_count()
+                x, it = solve(torch.from_numpy(f).cuda())
+                counts.append(amgh.launch_count() - n0)
+                iters.append(it)
+                assert np.linalg.norm(A @ x.cpu().numpy() - f) <= 2 * TOL * np.linalg.norm(f), (which, ctas)
+        finally:
+            amgh.debug_cluster_ctas(-1)
+        assert counts[0] == counts[2] == 1 and counts[1] > 1, (which, counts)
+        assert max(iters) - min(iters) <= 1, (which, iters)
+    # block mass solves: one cluster a column, or the replayed block loop
+    yd = torch.from_numpy(rng.standard_normal((3, p.sizes["n"]))).cuda()
+    sopts = dict(tol=1e-8, inner_tol=TOL, mass_tol=TOL)
+    u0, _, st0 = p.solve_block(yd, **sopts)
+    try:
+        amgh.debug_cluster_ctas(0)
+        u1, _, st1 = p.solve_block(yd, **sopts)
+    finally:
+        amgh.debug_cluster_ctas(-1)
+    assert st0 == 0 and st1 == 0
+    # two outer CGs to a relative residual of 1e-8 on a Hessian whose M_u-scaled condition number is below 1 / beta = 100
+    assert np.linalg.norm((u0 - u1).cpu().numpy()) <= 2e-6 * np.linalg.norm(u0.cpu().numpy())
+    p.close()
+
+
+def test_cluster_hook_rejects_bad_values():
+    from paper_2001_11533_gb300 import amgh
+    with pytest.raises(amgh.AmghError) as e:
+        amgh.debug_cluster_ctas(-2)
+    assert e.value.code == -1
