@@ -222,7 +222,7 @@ __device__ void cg_finalize(int mode, const double *t, CgScal *sc, double *out)
 
 // x = 0 (optional), r = f, reduce f.f ; host put tol^2 in sc->thr and maxit
 template <typename T>
-__global__ void k_cg_start(int n, const T *__restrict__ f, T *__restrict__ x, T *__restrict__ r, CgScal *sc,
+__global__ void k_cg_start(int n, const T *f, T *__restrict__ x, T *__restrict__ r, CgScal *sc,
                            int zero_x, double *partials, unsigned *ticket, int mode)
 {
     pdl_enter();
@@ -237,7 +237,7 @@ __global__ void k_cg_start(int n, const T *__restrict__ f, T *__restrict__ x, T 
 }
 
 // mass CG start: x = 0, r = f, z = invd r; reduce f.f
-__global__ void k_mass_start(int n, const double *__restrict__ f, double *__restrict__ x, double *__restrict__ r,
+__global__ void k_mass_start(int n, const double *f, double *__restrict__ x, double *__restrict__ r,
                              double *__restrict__ z, const double *__restrict__ invd, CgScal *sc, double *partials,
                              unsigned *ticket)
 {
@@ -256,19 +256,26 @@ __global__ void k_mass_start(int n, const double *__restrict__ f, double *__rest
 // K1: s = A z, reduce (r, z) and (z, s) -> alpha, beta.  z may be FP32 (the
 // output of an FP32 V-cycle) while A, r and s are FP64.
 template <typename T, typename Z, int TPR>
-__global__ void k_cg2_spmv(MatView<T> A, const Z *__restrict__ z, const T *__restrict__ r, T *__restrict__ s,
+__global__ void k_cg2_spmv(MatView<T> A, const Z *z, const T *r, T *__restrict__ s,
                            CgScal *sc, double *partials, unsigned *ticket)
 {
     int row = my_row<TPR>();
     RowPre<T> pre;
     PDL_ENTER_LOADING(&sc->done, (row_prefetch<T, TPR>(A, row, pre)))
-    T v = row_sum_pre<T, TPR>(A, row, pre, [&](int c) { return (T)__ldg(&z[c]); });
+    // row-local operands first, so their loads overlap the row's gathers
+    const bool lead = row < A.rows && row_leader<TPR>();
+    Z zr = 0;
+    T rr = 0;
+    if (lead) {
+        zr = z[row];
+        rr = r[row];
+    }
+    T v = row_sum_pre<T, TPR>(A, row, pre, [&](int c) { return (T)z[c]; });
     double a[2] = {0.0, 0.0}, tot[2];
-    if (row < A.rows && row_leader<TPR>()) {
+    if (lead) {
         s[row] = v;
-        double zr = (double)z[row];
-        a[0] = (double)r[row] * zr;
-        a[1] = zr * (double)v;
+        a[0] = (double)rr * (double)zr;
+        a[1] = (double)zr * (double)v;
     }
     if (reduce_last_block<2>(a, partials, ticket, tot)) cg_finalize(F_CG2, tot, sc, nullptr);
 }
@@ -276,20 +283,26 @@ __global__ void k_cg2_spmv(MatView<T> A, const Z *__restrict__ z, const T *__res
 // K1 with the products on the FP32 pipe: s = (A_hi + A_lo) z accumulated in
 // double-float (about 2^-48 relative), converted to FP64 per row
 template <typename Z, int TPR>
-__global__ void k_cg2_spmv_df(MatView<float> A, const float *__restrict__ lo, const Z *__restrict__ z,
-                              const double *__restrict__ r, double *__restrict__ s, CgScal *sc, double *partials,
+__global__ void k_cg2_spmv_df(MatView<float> A, const float *__restrict__ lo, const Z *z,
+                              const double *r, double *__restrict__ s, CgScal *sc, double *partials,
                               unsigned *ticket)
 {
     int row = my_row<TPR>();
     RowPreDf pre;
     PDL_ENTER_LOADING(&sc->done, row_prefetch_df<TPR>(A, lo, row, pre))
+    const bool lead = row < A.rows && row_leader<TPR>();
+    Z zr = 0;
+    double rr = 0.0;
+    if (lead) {
+        zr = z[row];
+        rr = r[row];
+    }
     double v = row_sum_df<Z, TPR>(A, lo, row, pre, z);
     double a[2] = {0.0, 0.0}, tot[2];
-    if (row < A.rows && row_leader<TPR>()) {
+    if (lead) {
         s[row] = v;
-        double zr = (double)z[row];
-        a[0] = r[row] * zr;
-        a[1] = zr * v;
+        a[0] = rr * (double)zr;
+        a[1] = (double)zr * v;
     }
     if (reduce_last_block<2>(a, partials, ticket, tot)) cg_finalize(F_CG2, tot, sc, nullptr);
 }
@@ -298,7 +311,7 @@ __global__ void k_cg2_spmv_df(MatView<float> A, const float *__restrict__ lo, co
 // optionally r32 = r (input of an FP32 V-cycle) or, for the Jacobi-
 // preconditioned mass CG, z = invd r for the next K1.
 template <typename T, typename Z>
-__global__ void k_cg2_update(int n, Z *__restrict__ z, const T *__restrict__ s, T *__restrict__ pv,
+__global__ void k_cg2_update(int n, Z *__restrict__ z, const T *s, T *__restrict__ pv,
                              T *__restrict__ q, T *__restrict__ x, T *__restrict__ r, float *__restrict__ r32,
                              const double *__restrict__ invd, T *__restrict__ vd, T *__restrict__ vx,
                              const T *__restrict__ vinvd, T c0, CgScal *sc, double *partials, unsigned *ticket)
@@ -311,7 +324,8 @@ __global__ void k_cg2_update(int n, Z *__restrict__ z, const T *__restrict__ s, 
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         T zi = (T)z[i];
         T pi = first ? zi : zi + b * pv[i];
-        T qi = first ? s[i] : s[i] + b * q[i];
+        T si = __ldcg(s + i); // a stream: read once
+        T qi = first ? si : si + b * q[i];
         pv[i] = pi;
         q[i] = qi;
         x[i] = x[i] + a * pi;
@@ -331,7 +345,7 @@ __global__ void k_cg2_update(int n, Z *__restrict__ z, const T *__restrict__ s, 
 
 // rz = r.z and p = z (first iteration) or beta from rz (later)
 template <typename T>
-__global__ void k_rz(int n, const T *__restrict__ r, const T *__restrict__ z, T *__restrict__ pv, CgScal *sc,
+__global__ void k_rz(int n, const T *r, const T *z, T *__restrict__ pv, CgScal *sc,
                      int first, double *partials, unsigned *ticket)
 {
     pdl_enter();
@@ -347,7 +361,7 @@ __global__ void k_rz(int n, const T *__restrict__ r, const T *__restrict__ z, T 
 
 // p = z + beta p
 template <typename T>
-__global__ void k_xpay(int n, const T *__restrict__ z, T *__restrict__ pv, const CgScal *sc)
+__global__ void k_xpay(int n, const T *z, T *__restrict__ pv, const CgScal *sc)
 {
     pdl_enter();
     SKIP_DONE();
@@ -356,8 +370,8 @@ __global__ void k_xpay(int n, const T *__restrict__ z, T *__restrict__ pv, const
 }
 
 // outer CG: x += alpha p, r -= alpha q, reduce r.r -> stop test
-__global__ void k_update(int n, double *__restrict__ x, double *__restrict__ r, const double *__restrict__ pv,
-                         const double *__restrict__ q, CgScal *sc, double *partials, unsigned *ticket)
+__global__ void k_update(int n, double *__restrict__ x, double *__restrict__ r, const double *pv,
+                         const double *q, CgScal *sc, double *partials, unsigned *ticket)
 {
     pdl_enter();
     SKIP_DONE();
@@ -373,7 +387,7 @@ __global__ void k_update(int n, double *__restrict__ x, double *__restrict__ r, 
 }
 
 // generic dot with finaliser (outer CG: p.Hp; r.z)
-__global__ void k_dot(int n, const double *__restrict__ x, const double *__restrict__ y, CgScal *sc, int mode,
+__global__ void k_dot(int n, const double *x, const double *y, CgScal *sc, int mode,
                       double *out, double *partials, unsigned *ticket)
 {
     pdl_enter();
@@ -384,7 +398,7 @@ __global__ void k_dot(int n, const double *__restrict__ x, const double *__restr
 }
 
 // refinement: r32 = r / scale
-__global__ void k_ref_to32(int n, const double *__restrict__ r, float *__restrict__ r32, const CgScal *rs)
+__global__ void k_ref_to32(int n, const double *r, float *__restrict__ r32, const CgScal *rs)
 {
     pdl_enter();
     if (rs->done) return;
@@ -394,7 +408,7 @@ __global__ void k_ref_to32(int n, const double *__restrict__ r, float *__restric
 }
 
 // refinement: y += scale * e
-__global__ void k_ref_add(int n, double *__restrict__ y, const float *__restrict__ e, const CgScal *rs)
+__global__ void k_ref_add(int n, double *__restrict__ y, const float *e, const CgScal *rs)
 {
     pdl_enter();
     if (rs->done) return;
@@ -405,13 +419,13 @@ __global__ void k_ref_add(int n, double *__restrict__ y, const float *__restrict
 
 // refinement: r = f - A y (FP64), reduce r.r -> stop test
 template <typename T, int TPR>
-__global__ void k_ref_resid(MatView<T> A, const T *__restrict__ f, const T *__restrict__ y, T *__restrict__ r,
+__global__ void k_ref_resid(MatView<T> A, const T *f, const T *y, T *__restrict__ r,
                             CgScal *rs, double *partials, unsigned *ticket)
 {
     pdl_enter();
     if (rs->done) return;
     int i = my_row<TPR>();
-    T ay = row_sum<T, TPR>(A, i, [&](int c) { return __ldg(&y[c]); });
+    T ay = row_sum<T, TPR>(A, i, [&](int c) { return y[c]; });
     double v[1] = {0.0}, tot[1];
     if (i < A.rows && row_leader<TPR>()) {
         T ri = f[i] - ay;
@@ -433,7 +447,7 @@ __global__ void k_set_scal(CgScal *sc, double tol2, int maxit)
     sc->status = CG_RUNNING;
 }
 
-__global__ void k_axpby(int n, double a, const double *__restrict__ x, double b, const double *__restrict__ y,
+__global__ void k_axpby(int n, double a, const double *x, double b, const double *y,
                         double *__restrict__ out)
 {
     pdl_enter();
@@ -691,7 +705,7 @@ int vec_fill(amgh_problem *p, int n, double v, double *x)
 // ||f||^2 -> sc->scale, the power of two nearest 1 / ||f||.  The double-float
 // CG solves for the scaled right side (an exact scaling) so that its FP32
 // halves stay far from the FP32 exponent limits whatever the size of f.
-__global__ void k_df_norm(int n, const double *__restrict__ f, CgScal *sc, double *partials, unsigned *ticket)
+__global__ void k_df_norm(int n, const double *f, CgScal *sc, double *partials, unsigned *ticket)
 {
     pdl_enter();
     double v[1] = {0.0}, tot[1];
@@ -700,7 +714,7 @@ __global__ void k_df_norm(int n, const double *__restrict__ f, CgScal *sc, doubl
 }
 
 // r = scale f (split into hi/lo), x = 0, reduce (scale f).(scale f)
-__global__ void k_df_start(int n, const double *__restrict__ f, float *__restrict__ xh, float *__restrict__ xl,
+__global__ void k_df_start(int n, const double *f, float *__restrict__ xh, float *__restrict__ xl,
                            float *__restrict__ rh, float *__restrict__ rl, CgScal *sc, double *partials,
                            unsigned *ticket)
 {
@@ -725,8 +739,8 @@ __global__ void k_df_start(int n, const double *__restrict__ f, float *__restric
 // the wait for the kernel before (PDL_ENTER_LOADING); the walking form keeps
 // the fewer registers (48 against 64) that its occupancy needs.
 template <int TPR, bool PRE>
-__global__ void k_df_spmv(MatView<float> A, const float *__restrict__ lo, const float *__restrict__ z,
-                          const float *__restrict__ rh, const float *__restrict__ rl, float *__restrict__ sh,
+__global__ void k_df_spmv(MatView<float> A, const float *__restrict__ lo, const float *z,
+                          const float *rh, const float *rl, float *__restrict__ sh,
                           float *__restrict__ sl, CgScal *sc, double *partials, unsigned *ticket)
 {
     RowPreDf pre;
@@ -767,7 +781,7 @@ __global__ void k_df_spmv(MatView<float> A, const float *__restrict__ lo, const 
 // With invd32 the preconditioner is Jacobi and the new z = D^-1 r (FP32, from
 // r's hi half) is written over z in the same pass (element i is read before it
 // is written, by the same thread).
-__global__ void k_df_update(int n, const float *z, const float *__restrict__ sh, const float *__restrict__ sl,
+__global__ void k_df_update(int n, const float *z, const float *sh, const float *sl,
                             float *__restrict__ ph, float *__restrict__ pl, float *__restrict__ qh,
                             float *__restrict__ ql, float *__restrict__ xh, float *__restrict__ xl,
                             float *__restrict__ rh, float *__restrict__ rl, const float *__restrict__ invd32,
@@ -787,8 +801,8 @@ __global__ void k_df_update(int n, const float *z, const float *__restrict__ sh,
     };
     auto load = [&](int i, In &e) {
         e.z = z[i];
-        e.s1 = sh[i];
-        e.s2 = sl[i];
+        e.s1 = __ldcg(sh + i); // a stream: read once
+        e.s2 = __ldcg(sl + i);
         e.p1 = ph[i];
         e.p2 = pl[i];
         e.q1 = qh[i];
@@ -840,7 +854,7 @@ __global__ void k_df_update(int n, const float *z, const float *__restrict__ sh,
 }
 
 // y = x / scale (exact: scale is a power of two)
-__global__ void k_df_to_double(int n, const float *__restrict__ xh, const float *__restrict__ xl,
+__global__ void k_df_to_double(int n, const float *xh, const float *xl,
                                const CgScal *sc, double *__restrict__ y)
 {
     pdl_enter();
@@ -922,7 +936,7 @@ int dfcg_update(amgh_problem *p, RedSlot &red, int n, const float *z, const doub
 }
 
 // z = D^-1 r from r's hi half (Jacobi start of the double-float mass CG)
-__global__ void k_df_jacobi(int n, const float *__restrict__ rh, const float *__restrict__ invd32,
+__global__ void k_df_jacobi(int n, const float *rh, const float *__restrict__ invd32,
                             float *__restrict__ z)
 {
     pdl_enter();

@@ -97,48 +97,6 @@ __device__ __forceinline__ void ldk(const double *p, double (&v)[K])
     }
 }
 
-// read-only gathers (the source is not written by the same kernel)
-template <int K>
-__device__ __forceinline__ void ldk_ro(const float *p, float (&v)[K])
-{
-    if constexpr (K % 4 == 0) {
-#pragma unroll
-        for (int i = 0; i < K / 4; i++) {
-            float4 w = __ldg(reinterpret_cast<const float4 *>(p) + i);
-            v[4 * i] = w.x;
-            v[4 * i + 1] = w.y;
-            v[4 * i + 2] = w.z;
-            v[4 * i + 3] = w.w;
-        }
-    } else if constexpr (K % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < K / 2; i++) {
-            float2 w = __ldg(reinterpret_cast<const float2 *>(p) + i);
-            v[2 * i] = w.x;
-            v[2 * i + 1] = w.y;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < K; i++) v[i] = __ldg(p + i);
-    }
-}
-
-template <int K>
-__device__ __forceinline__ void ldk_ro(const double *p, double (&v)[K])
-{
-    if constexpr (K % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < K / 2; i++) {
-            double2 w = __ldg(reinterpret_cast<const double2 *>(p) + i);
-            v[2 * i] = w.x;
-            v[2 * i + 1] = w.y;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < K; i++) v[i] = __ldg(p + i);
-    }
-}
-
 // loads through L2 (ld.global.cg): vectors that other blocks of the same
 // launch have written (the persistent kernel; L1 is not coherent across SMs)
 template <int K>
@@ -205,7 +163,7 @@ struct Chunk {
 
 // row of A times K columns of x; every lane of the group returns the K sums
 template <typename T, int TPR, int K>
-__device__ __forceinline__ void row_sum_k(const MatView<T> &m, int row, const T *__restrict__ x, T (&acc)[K])
+__device__ __forceinline__ void row_sum_k(const MatView<T> &m, int row, const T *x, T (&acc)[K])
 {
     constexpr int STEP = TPR == 1 ? 32 : TPR;
     constexpr int U = Chunk<T, K>::U;
@@ -228,7 +186,7 @@ __device__ __forceinline__ void row_sum_k(const MatView<T> &m, int row, const T 
                 T xv[U][K];
 #pragma unroll
                 for (int j = 0; j < U; j++) {
-                    if (cc[j0 + j] >= 0) ldk_ro<K>(x + (int64_t)cc[j0 + j] * K, xv[j]);
+                    if (cc[j0 + j] >= 0) ldk<K>(x + (int64_t)cc[j0 + j] * K, xv[j]);
                     else {
 #pragma unroll
                         for (int c = 0; c < K; c++) xv[j][c] = (T)0;
@@ -246,7 +204,7 @@ __device__ __forceinline__ void row_sum_k(const MatView<T> &m, int row, const T 
             for (; k < end; k += STEP) {
                 T a = m.v[k];
                 T xv[K];
-                ldk_ro<K>(x + (int64_t)col_of(m, row, k) * K, xv);
+                ldk<K>(x + (int64_t)col_of(m, row, k) * K, xv);
 #pragma unroll
                 for (int c = 0; c < K; c++) acc[c] = rfma(a, xv[c], acc[c]);
             }
@@ -265,7 +223,7 @@ __device__ __forceinline__ void row_sum_k(const MatView<T> &m, int row, const T 
 // every lane of the group returns the K normalised sums
 template <typename Z, int TPR, int K, bool CG = false>
 __device__ __forceinline__ void row_sum_df_k(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             const Z *__restrict__ z, DF (&out)[K])
+                                             const Z *z, DF (&out)[K])
 {
     // CG: z is written by other blocks of the same launch: gathers through L2
     constexpr int STEP = TPR == 1 ? 32 : TPR;
@@ -294,7 +252,7 @@ __device__ __forceinline__ void row_sum_df_k(const MatView<float> &m, const floa
                 for (int j = 0; j < U; j++) {
                     if (cc[j0 + j] >= 0) {
                         if constexpr (CG) ldk_cg<K>(z + (int64_t)cc[j0 + j] * K, zv[j]);
-                        else ldk_ro<K>(z + (int64_t)cc[j0 + j] * K, zv[j]);
+                        else ldk<K>(z + (int64_t)cc[j0 + j] * K, zv[j]);
                     } else {
 #pragma unroll
                         for (int c = 0; c < K; c++) zv[j][c] = (Z)0;
@@ -313,7 +271,7 @@ __device__ __forceinline__ void row_sum_df_k(const MatView<float> &m, const floa
                 float ah = m.v[k], al = lo[k];
                 Z zv[K];
                 if constexpr (CG) ldk_cg<K>(z + (int64_t)col_of(m, row, k) * K, zv);
-                else ldk_ro<K>(z + (int64_t)col_of(m, row, k) * K, zv);
+                else ldk<K>(z + (int64_t)col_of(m, row, k) * K, zv);
 #pragma unroll
                 for (int c = 0; c < K; c++) df_term<Z>(acc[c], ah, al, zv[c]);
             }
@@ -591,7 +549,7 @@ __device__ void fin_rr(BScal *bs, const double *t)
 // ------------------------------------------------------------------ CG kernels
 // x = 0, r = f, optionally z = invd f (Jacobi, in the type Z of z); f.f per column
 template <typename Z, int K>
-__global__ void kb_cg_start(int n, const double *__restrict__ f, double *__restrict__ x, double *__restrict__ r,
+__global__ void kb_cg_start(int n, const double *f, double *__restrict__ x, double *__restrict__ r,
                             Z *__restrict__ z, const double *__restrict__ invd, BScal *bs, double tol2,
                             int maxit, double *partials, unsigned *ticket)
 {
@@ -624,7 +582,7 @@ __global__ void kb_cg_start(int n, const double *__restrict__ f, double *__restr
 // s = A z with (r, z) and (z, s) per column -> alpha, beta, in FP64 (precision 0,
 // as the single-column FP64 CG)
 template <int TPR, int K>
-__global__ void kb_cg_spmv64(MatView<double> A, const double *__restrict__ z, const double *__restrict__ r,
+__global__ void kb_cg_spmv64(MatView<double> A, const double *z, const double *r,
                              double *__restrict__ s, BScal *bs, double *partials, unsigned *ticket)
 {
     pdl_enter();
@@ -640,7 +598,7 @@ __global__ void kb_cg_spmv64(MatView<double> A, const double *__restrict__ z, co
         int64_t o = (int64_t)row * K;
         stk<K>(s + o, sv);
         double zr[K], rr[K];
-        ldk_ro<K>(z + o, zr);
+        ldk<K>(z + o, zr);
         ldk<K>(r + o, rr);
 #pragma unroll
         for (int c = 0; c < K; c++) {
@@ -655,7 +613,7 @@ __global__ void kb_cg_spmv64(MatView<double> A, const double *__restrict__ z, co
 // r -= alpha q per running column; for Jacobi z = invd r; r.r per column.
 // For K = 8 two threads share a row, four columns each.
 template <typename Z, int K>
-__global__ void kb_cg_update(int n, Z *z, const double *__restrict__ s, double *__restrict__ pv,
+__global__ void kb_cg_update(int n, Z *z, const double *s, double *__restrict__ pv,
                              double *__restrict__ q, double *__restrict__ x, double *__restrict__ r,
                              const double *__restrict__ invd, BScal *bs, double *partials,
                              unsigned *ticket)
@@ -750,7 +708,7 @@ __device__ __forceinline__ double inv_pow2(double s)
 
 // f.f per column (FP64, once per solve) -> scale and the scaled threshold
 template <int K>
-__global__ void kbd_norm(int n, const double *__restrict__ f, BScal *bs, double tol2, int maxit,
+__global__ void kbd_norm(int n, const double *f, BScal *bs, double tol2, int maxit,
                          double *partials, unsigned *ticket)
 {
     pdl_enter();
@@ -769,7 +727,7 @@ __global__ void kbd_norm(int n, const double *__restrict__ f, BScal *bs, double 
 
 // r = scale_c f (split into hi/lo), x = 0; for Jacobi also z = invd r_hi
 template <int K>
-__global__ void kbd_start(int64_t nk, const double *__restrict__ f, float *__restrict__ xh, float *__restrict__ xl,
+__global__ void kbd_start(int64_t nk, const double *f, float *__restrict__ xh, float *__restrict__ xl,
                           float *__restrict__ rh, float *__restrict__ rl, float *__restrict__ z,
                           const float *__restrict__ invd32, const BScal *bs)
 {
@@ -789,8 +747,8 @@ __global__ void kbd_start(int64_t nk, const double *__restrict__ f, float *__res
 // per column -> alpha, beta
 template <int TPR, int K>
 __global__ void __launch_bounds__(TPB_K, 3) kbd_spmv(MatView<float> A, const float *__restrict__ lo,
-                                                     const float *__restrict__ z, const float *__restrict__ rh,
-                                                     const float *__restrict__ rl, float *__restrict__ sh,
+                                                     const float *z, const float *rh,
+                                                     const float *rl, float *__restrict__ sh,
                                                      float *__restrict__ sl, BScal *bs, double *partials,
                                                      unsigned *ticket)
 {
@@ -813,7 +771,7 @@ __global__ void __launch_bounds__(TPB_K, 3) kbd_spmv(MatView<float> A, const flo
         }
         stk<K>(sh + o, h);
         stk<K>(sl + o, l);
-        ldk_ro<K>(z + o, zr);
+        ldk<K>(z + o, zr);
         ldk<K>(rh + o, rhv);
         ldk<K>(rl + o, rlv);
 #pragma unroll
@@ -829,7 +787,7 @@ __global__ void __launch_bounds__(TPB_K, 3) kbd_spmv(MatView<float> A, const flo
 // column in double-float; with invd32 (Jacobi) z = invd r_hi; r.r per column.
 // For K = 8 two threads share a row, four columns each.
 template <int K>
-__global__ void kbd_update(int n, float *z, const float *__restrict__ sh, const float *__restrict__ sl,
+__global__ void kbd_update(int n, float *z, const float *sh, const float *sl,
                            float *__restrict__ ph, float *__restrict__ pl, float *__restrict__ qh,
                            float *__restrict__ ql, float *__restrict__ xh, float *__restrict__ xl,
                            float *__restrict__ rh, float *__restrict__ rl, const float *__restrict__ invd32,
@@ -920,7 +878,7 @@ __global__ void kbd_update(int n, float *z, const float *__restrict__ sh, const 
 
 // x = (x_hi + x_lo) / scale_c (FP64, once per solve)
 template <int K>
-__global__ void kbd_out(int64_t nk, const float *__restrict__ xh, const float *__restrict__ xl, const BScal *bs,
+__global__ void kbd_out(int64_t nk, const float *xh, const float *xl, const BScal *bs,
                         double *__restrict__ y)
 {
     pdl_enter();
@@ -1074,7 +1032,7 @@ __global__ void __launch_bounds__(TPB_K) kbp_mass_cg(MatView<float> A, const flo
 // ------------------------------------------------------------------ V-cycle kernels
 // first smoother step from zero: d = x = c D^-1 b
 template <typename T, int K>
-__global__ void kb_cheb_first(int n, const T *__restrict__ invd, const T *__restrict__ b, T *__restrict__ d,
+__global__ void kb_cheb_first(int n, const T *__restrict__ invd, const T *b, T *__restrict__ d,
                               T *__restrict__ x, T cf, const BScal *bs)
 {
     pdl_enter();
@@ -1093,8 +1051,8 @@ __global__ void kb_cheb_first(int n, const T *__restrict__ invd, const T *__rest
 
 // Chebyshev step: d' = c_d d + c_r D^-1 (b - A x), x' = x + d'
 template <typename T, int TPR, int K>
-__global__ void kb_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *__restrict__ b,
-                             const T *__restrict__ x, T *__restrict__ d, T *__restrict__ xn, T cdv, T crv,
+__global__ void kb_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *b,
+                             const T *x, T *__restrict__ d, T *__restrict__ xn, T cdv, T crv,
                              const BScal *bs)
 {
     pdl_enter();
@@ -1118,7 +1076,7 @@ __global__ void kb_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *
 
 // r = b - A x
 template <typename T, int TPR, int K>
-__global__ void kb_residual(MatView<T> A, const T *__restrict__ b, const T *__restrict__ x, T *__restrict__ r,
+__global__ void kb_residual(MatView<T> A, const T *b, const T *x, T *__restrict__ r,
                             const BScal *bs)
 {
     pdl_enter();
@@ -1138,7 +1096,7 @@ __global__ void kb_residual(MatView<T> A, const T *__restrict__ b, const T *__re
 
 // y = A x (add = 0) or y += A x (add = 1): restriction and prolongation
 template <typename T, int TPR, int K>
-__global__ void kb_apply(MatView<T> A, const T *__restrict__ x, T *__restrict__ y, int add, const BScal *bs)
+__global__ void kb_apply(MatView<T> A, const T *x, T *__restrict__ y, int add, const BScal *bs)
 {
     pdl_enter();
     if (bs && bs->all) return;
@@ -1160,7 +1118,7 @@ __global__ void kb_apply(MatView<T> A, const T *__restrict__ x, T *__restrict__ 
 // x = inv b for a dense row-major inverse with leading dimension ld: one warp
 // per row
 template <typename T, int K>
-__global__ void kb_dense(int n, const T *__restrict__ inv, int ld, const T *__restrict__ b, T *__restrict__ x,
+__global__ void kb_dense(int n, const T *__restrict__ inv, int ld, const T *b, T *__restrict__ x,
                          const BScal *bs)
 {
     pdl_enter();
@@ -1174,7 +1132,7 @@ __global__ void kb_dense(int n, const T *__restrict__ inv, int ld, const T *__re
     for (int c = 0; c < K; c++) acc[c] = (T)0;
     for (int j = lane; j < n; j += 32) {
         T aj = a[j], bv[K];
-        ldk_ro<K>(b + (int64_t)j * K, bv);
+        ldk<K>(b + (int64_t)j * K, bv);
 #pragma unroll
         for (int c = 0; c < K; c++) acc[c] = rfma(aj, bv[c], acc[c]);
     }
@@ -1187,7 +1145,7 @@ __global__ void kb_dense(int n, const T *__restrict__ inv, int ld, const T *__re
 }
 
 template <typename T>
-__global__ void kb_copy(int64_t nk, const T *__restrict__ a, T *__restrict__ b, const BScal *bs)
+__global__ void kb_copy(int64_t nk, const T *a, T *__restrict__ b, const BScal *bs)
 {
     pdl_enter();
     if (bs && bs->all) return;
@@ -1198,7 +1156,7 @@ __global__ void kb_copy(int64_t nk, const T *__restrict__ a, T *__restrict__ b, 
 // ------------------------------------------------------------------ FP64 operators and vectors
 // y = alpha A x + beta y (beta = 0: y is not read)
 template <int TPR, int K>
-__global__ void kb_spmm(MatView<double> A, const double *__restrict__ x, double *__restrict__ y, double alpha,
+__global__ void kb_spmm(MatView<double> A, const double *x, double *__restrict__ y, double alpha,
                         double beta)
 {
     pdl_enter();
@@ -1227,7 +1185,7 @@ struct Coef {
 
 // out = a_c x + b_c y per column (y may be null)
 template <int K>
-__global__ void kb_axpby(int n, Coef cf, const double *__restrict__ x, const double *__restrict__ y, double *out)
+__global__ void kb_axpby(int n, Coef cf, const double *x, const double *y, double *out)
 {
     pdl_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1249,8 +1207,8 @@ __global__ void kb_axpby(int n, Coef cf, const double *__restrict__ x, const dou
 
 // out = ta + (w1 - tb) / beta (the two-grid combination of Eq.
 // twogridinmultiactual, all columns)
-__global__ void kb_rcomb(int64_t nk, const double *__restrict__ ta, const double *__restrict__ w1,
-                         const double *__restrict__ tb, double beta, double *__restrict__ out)
+__global__ void kb_rcomb(int64_t nk, const double *ta, const double *w1,
+                         const double *tb, double beta, double *__restrict__ out)
 {
     pdl_enter();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nk; i += (int64_t)gridDim.x * blockDim.x)
@@ -1259,7 +1217,7 @@ __global__ void kb_rcomb(int64_t nk, const double *__restrict__ ta, const double
 
 // out[c] = (x_c, y_c)
 template <int K>
-__global__ void kb_dot(int n, const double *__restrict__ x, const double *__restrict__ y, double *out,
+__global__ void kb_dot(int n, const double *x, const double *y, double *out,
                        double *partials, unsigned *ticket)
 {
     pdl_enter();
@@ -1281,7 +1239,7 @@ __global__ void kb_dot(int n, const double *__restrict__ x, const double *__rest
 // column-major (leading dimension ld, nc columns) -> interleaved K columns,
 // padding columns zero
 template <int K>
-__global__ void kb_pack(int n, int nc, const double *__restrict__ src, int64_t ld, double *__restrict__ dst)
+__global__ void kb_pack(int n, int nc, const double *src, int64_t ld, double *__restrict__ dst)
 {
     pdl_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1293,7 +1251,7 @@ __global__ void kb_pack(int n, int nc, const double *__restrict__ src, int64_t l
 }
 
 template <int K>
-__global__ void kb_unpack(int n, int nc, const double *__restrict__ src, double *__restrict__ dst, int64_t ld)
+__global__ void kb_unpack(int n, int nc, const double *src, double *__restrict__ dst, int64_t ld)
 {
     pdl_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1307,7 +1265,7 @@ __global__ void kb_unpack(int n, int nc, const double *__restrict__ src, double 
 
 // desired states at the state dofs: dst[s][c] = yd[c][vertex_of_state[s]]
 template <int K>
-__global__ void kb_gather_state(int m, int nc, const double *__restrict__ yd, int64_t nv,
+__global__ void kb_gather_state(int m, int nc, const double *yd, int64_t nv,
                                 const int *__restrict__ vos, double *__restrict__ dst)
 {
     pdl_enter();

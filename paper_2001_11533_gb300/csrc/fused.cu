@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(FUSE_TPB, 1)
 // blocks, all resident at once, phases separated by grid_sync
 __global__ void __launch_bounds__(FUSE_TPB, 1)
     k_vcycle_grid(const FusedCycle *__restrict__ fc, const float *b0, float *x0, int preinit,
-                  const int *__restrict__ skip, GridBar *gb)
+                  const int *skip, GridBar *gb)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (skip && *skip) return; // uniform: the flag is not written while this kernel runs

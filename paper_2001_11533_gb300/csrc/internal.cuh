@@ -56,6 +56,12 @@ void amgh_set_capturing(int on);
 // place from them; grids above 608 blocks used to hold it back, which cost
 // 0.5 % of the 1025^2 L-shape's step.)  Without the launch attribute the wait
 // returns at once.
+//
+// Vectors that a kernel before may write are read with ordinary loads, through
+// pointers that are not const __restrict__: read-only loads (ld.global.nc, which
+// __ldg and const __restrict__ stand for) promise data that does not change
+// while the kernel is resident, and a kernel scheduled early is resident while
+// its predecessor writes.  They are kept for what the setup wrote.
 __device__ __forceinline__ void pdl_enter()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -84,7 +84,7 @@ __host__ __device__ constexpr int kuhn_nbr(int di, int dj, int dk)
 // the 6 neighbour values are loaded together and combined in a fixed order.
 template <typename T, typename K>
 __device__ __forceinline__ T kuhn_row(int N, T h6, const K *__restrict__ kappa, const int *__restrict__ sov,
-                                      const int *__restrict__ vos, const T *__restrict__ x, int r)
+                                      const int *__restrict__ vos, const T *x, int r)
 {
     const int64_t v = vos[r];
     const int i = (int)(v % N), j = (int)((v / N) % N), k = (int)(v / ((int64_t)N * N));
@@ -151,9 +151,9 @@ __global__ void k_kuhn_apply(int m, int N, T h6, const K *__restrict__ kappa, co
 // Chebyshev step of the level-0 smoother with the matrix-free operator:
 // d' = c_d d + c_r D^-1 (b - A x), x' = x + d'
 __global__ void k_kuhn_cheb(int m, int N, float h6, const float *__restrict__ kappa, const int *__restrict__ sov,
-                            const int *__restrict__ vos, const float *__restrict__ invd, const float *__restrict__ b,
-                            const float *__restrict__ x, float *__restrict__ d, float *__restrict__ xn, float cdv,
-                            float crv, const int *__restrict__ skip)
+                            const int *__restrict__ vos, const float *__restrict__ invd, const float *b,
+                            const float *x, float *__restrict__ d, float *__restrict__ xn, float cdv,
+                            float crv, const int *skip)
 {
     pdl_enter();
     if (skip && *skip) return;
@@ -168,8 +168,8 @@ __global__ void k_kuhn_cheb(int m, int N, float h6, const float *__restrict__ ka
 }
 
 __global__ void k_kuhn_residual(int m, int N, float h6, const float *__restrict__ kappa, const int *__restrict__ sov,
-                                const int *__restrict__ vos, const float *__restrict__ b, const float *__restrict__ x,
-                                float *__restrict__ res, const int *__restrict__ skip)
+                                const int *__restrict__ vos, const float *b, const float *x,
+                                float *__restrict__ res, const int *skip)
 {
     pdl_enter();
     if (skip && *skip) return;

@@ -148,7 +148,7 @@ struct VBuf<float> {
 };
 
 template <typename T>
-__global__ void k_copy(int n, const T *__restrict__ a, T *__restrict__ b, const int *skip)
+__global__ void k_copy(int n, const T *a, T *__restrict__ b, const int *skip)
 {
     pdl_enter();
     if (skip && *skip) return;
@@ -675,8 +675,8 @@ int hessian_level(amgh_problem *p, int l, const double *v, double *hv)
 }
 
 // ------------------------------------------------------------------ MLAS
-__global__ void k_r_combine(int n, const double *__restrict__ ta, const double *__restrict__ w1,
-                            const double *__restrict__ tb, double beta, double *__restrict__ out)
+__global__ void k_r_combine(int n, const double *ta, const double *w1,
+                            const double *tb, double beta, double *__restrict__ out)
 {
     pdl_enter();
     int i = blockIdx.x * blockDim.x + threadIdx.x;

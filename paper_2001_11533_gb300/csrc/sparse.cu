@@ -458,34 +458,34 @@ int build_lo_parts(Arena &ar, DevCsr &a, cudaStream_t s)
     if (skip && *skip) return
 
 template <typename T, int TPR>
-__global__ void k_spmv(MatView<T> A, const T *__restrict__ x, T *__restrict__ y, const int *__restrict__ skip)
+__global__ void k_spmv(MatView<T> A, const T *x, T *__restrict__ y, const int *skip)
 {
     int r = my_row<TPR>();
     RowPre<T> pre;
     PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pre)))
-    T v = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return __ldg(&x[c]); });
+    T v = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return x[c]; });
     if (r < A.rows && row_leader<TPR>()) y[r] = v;
 }
 
 // y = A1 x1 + c A2 x2
 template <typename T, int TPR>
-__global__ void k_spmv2(MatView<T> A1, const T *__restrict__ x1, MatView<T> A2, const T *__restrict__ x2, T c,
-                        T *__restrict__ y, const int *__restrict__ skip)
+__global__ void k_spmv2(MatView<T> A1, const T *x1, MatView<T> A2, const T *x2, T c,
+                        T *__restrict__ y, const int *skip)
 {
     pdl_enter();
     SKIP_RETURN();
     int r = my_row<TPR>();
-    T a = row_sum<T, TPR>(A1, r, [&](int j) { return __ldg(&x1[j]); });
+    T a = row_sum<T, TPR>(A1, r, [&](int j) { return x1[j]; });
     // A2 may use another layout; it is read row-wise by the group leader's lanes
-    T b = row_sum<T, TPR>(A2, r, [&](int j) { return __ldg(&x2[j]); });
+    T b = row_sum<T, TPR>(A2, r, [&](int j) { return x2[j]; });
     if (r < A1.rows && row_leader<TPR>()) y[r] = a + c * b;
 }
 
 // smoother step: d = cd d + cr D^-1 (b - A x); xn = x + d
 template <typename T, int TPR>
-__global__ void k_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *__restrict__ b,
-                            const T *__restrict__ x, T *__restrict__ d, T *__restrict__ xn, T cdv, T crv,
-                            const int *__restrict__ skip)
+__global__ void k_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *b,
+                            const T *x, T *__restrict__ d, T *__restrict__ xn, T cdv, T crv,
+                            const int *skip)
 {
     int r = my_row<TPR>();
     bool lead = r < A.rows && row_leader<TPR>();
@@ -499,7 +499,7 @@ __global__ void k_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *_
         dr = d[r];
         xr = x[r];
     }
-    T ax = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return __ldg(&x[c]); });
+    T ax = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return x[c]; });
     if (lead) {
         T dn, xv;
         cheb_point(br, ax, ir, dr, xr, cdv, crv, dn, xv);
@@ -510,8 +510,8 @@ __global__ void k_cheb_step(MatView<T> A, const T *__restrict__ invd, const T *_
 
 // first smoother step from x = 0: d = c D^-1 b; x = d
 template <typename T>
-__global__ void k_cheb_first(int n, const T *__restrict__ invd, const T *__restrict__ b, T *__restrict__ d,
-                             T *__restrict__ x, T c, const int *__restrict__ skip)
+__global__ void k_cheb_first(int n, const T *__restrict__ invd, const T *b, T *__restrict__ d,
+                             T *__restrict__ x, T c, const int *skip)
 {
     pdl_enter();
     SKIP_RETURN();
@@ -547,8 +547,8 @@ __device__ int g_bulk_first_polls = BULK_POLLS;
 template <bool D16>
 __global__ void __launch_bounds__(32 * ELL_SLICES)
     k_cheb_step_ell(int rows, int nslices, int W, const float *__restrict__ v, const void *__restrict__ cols,
-                    const float *__restrict__ invd, const float *__restrict__ b, const float *__restrict__ x,
-                    float *__restrict__ d, float *__restrict__ xn, float cdv, float crv, const int *__restrict__ skip)
+                    const float *__restrict__ invd, const float *b, const float *x,
+                    float *__restrict__ d, float *__restrict__ xn, float cdv, float crv, const int *skip)
 {
     extern __shared__ __align__(16) unsigned char ell_sm[];
     __shared__ __align__(8) uint64_t bar;
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(32 * ELL_SLICES)
         if (j < W) {
             int k = base + 32 * j;
             int c = D16 ? row + (int)((const short *)sc)[k] : ((const int *)sc)[k];
-            xv[j] = __ldg(&x[c]);
+            xv[j] = x[c];
         }
     }
     float ax = 0.f;
@@ -614,31 +614,31 @@ __global__ void __launch_bounds__(32 * ELL_SLICES)
 }
 
 template <typename T, int TPR>
-__global__ void k_residual(MatView<T> A, const T *__restrict__ b, const T *__restrict__ x, T *__restrict__ res,
-                           const int *__restrict__ skip)
+__global__ void k_residual(MatView<T> A, const T *b, const T *x, T *__restrict__ res,
+                           const int *skip)
 {
     int r = my_row<TPR>();
     bool lead = r < A.rows && row_leader<TPR>();
     RowPre<T> pre;
     PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pre)))
     T br = lead ? b[r] : (T)0;
-    T ax = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return __ldg(&x[c]); });
+    T ax = row_sum_pre<T, TPR>(A, r, pre, [&](int c) { return x[c]; });
     if (lead) res[r] = rsub(br, ax);
 }
 
 // restriction b_c = S^T r fused with the first smoother step of the coarse
 // level from zero: d_c = x_c = c0 D_c^-1 b_c
 template <typename T, int TPR>
-__global__ void k_restrict_first(MatView<T> St, const T *__restrict__ r, T *__restrict__ bc,
+__global__ void k_restrict_first(MatView<T> St, const T *r, T *__restrict__ bc,
                                  const T *__restrict__ invd, T *__restrict__ d, T *__restrict__ x, T c0,
-                                 const int *__restrict__ skip)
+                                 const int *skip)
 {
     int i = my_row<TPR>();
     bool lead = i < St.rows && row_leader<TPR>();
     RowPre<T> pre;
     T ir = 0;
     PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(St, i, pre)); ir = lead ? invd[i] : (T)0)
-    T b = row_sum_pre<T, TPR>(St, i, pre, [&](int c) { return __ldg(&r[c]); });
+    T b = row_sum_pre<T, TPR>(St, i, pre, [&](int c) { return r[c]; });
     if (lead) {
         bc[i] = b;
         T v = cheb_first_point(b, ir, c0);
@@ -648,22 +648,22 @@ __global__ void k_restrict_first(MatView<T> St, const T *__restrict__ r, T *__re
 }
 
 template <typename T, int TPR>
-__global__ void k_prolong_add(MatView<T> S, const T *__restrict__ e, T *__restrict__ x,
-                              const int *__restrict__ skip)
+__global__ void k_prolong_add(MatView<T> S, const T *e, T *__restrict__ x,
+                              const int *skip)
 {
     int i = my_row<TPR>();
     bool lead = i < S.rows && row_leader<TPR>();
     RowPre<T> pre;
     PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(S, i, pre)))
     T xi = lead ? x[i] : (T)0;
-    T v = row_sum_pre<T, TPR>(S, i, pre, [&](int c) { return __ldg(&e[c]); });
+    T v = row_sum_pre<T, TPR>(S, i, pre, [&](int c) { return e[c]; });
     if (lead) x[i] = radd(xi, v);
 }
 
 // x = inv b, one warp per row of the dense explicit inverse
 template <typename T>
-__global__ void k_dense_gemv(int n, const double *__restrict__ inv, const T *__restrict__ b, T *__restrict__ x,
-                             const int *__restrict__ skip)
+__global__ void k_dense_gemv(int n, const double *__restrict__ inv, const T *b, T *__restrict__ x,
+                             const int *skip)
 {
     pdl_enter();
     SKIP_RETURN();
@@ -679,8 +679,8 @@ __global__ void k_dense_gemv(int n, const double *__restrict__ inv, const T *__r
 // FP32 copy, one warp per row, 16-byte loads of the padded row and (VEC) of
 // b (the last partial group of four read element by element)
 template <bool VEC>
-__global__ void k_dense_gemv32(int n, int ld, const float *__restrict__ inv, const float *__restrict__ b,
-                               float *__restrict__ x, const int *__restrict__ skip)
+__global__ void k_dense_gemv32(int n, int ld, const float *__restrict__ inv, const float *b,
+                               float *__restrict__ x, const int *skip)
 {
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     DensePre pre;
@@ -911,13 +911,13 @@ int spmv2(amgh_problem *p, const DevCsr &a1, const double *x1, const DevCsr &a2,
 
 // y = A x + c y  (used when the two operands of spmv2 have different layouts)
 template <typename T, int TPR>
-__global__ void k_spmv_axpy(MatView<T> A, const T *__restrict__ x, T c, T *__restrict__ y,
-                            const int *__restrict__ skip)
+__global__ void k_spmv_axpy(MatView<T> A, const T *x, T c, T *__restrict__ y,
+                            const int *skip)
 {
     pdl_enter();
     SKIP_RETURN();
     int r = my_row<TPR>();
-    T v = row_sum<T, TPR>(A, r, [&](int j) { return __ldg(&x[j]); });
+    T v = row_sum<T, TPR>(A, r, [&](int j) { return x[j]; });
     if (r < A.rows && row_leader<TPR>()) y[r] = v + c * y[r];
 }
 

@@ -373,15 +373,15 @@ __device__ __forceinline__ DF row_sum_df_xf(const MatView<float> &m, const float
 
 template <typename Z, int TPR>
 __device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             RowPreDf &p, const Z *__restrict__ z)
+                                             RowPreDf &p, const Z *z)
 {
-    return row_sum_df_xf<Z, TPR>(m, lo, row, p, [&](int c) { return __ldg(&z[c]); });
+    return row_sum_df_xf<Z, TPR>(m, lo, row, p, [&](int c) { return z[c]; });
 }
 
 // sum_j a_rj z_j in double-float (normalised)
 template <typename Z, int TPR>
 __device__ __forceinline__ DF row_sum_dfv(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                          RowPreDf &p, const Z *__restrict__ z)
+                                          RowPreDf &p, const Z *z)
 {
     DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, p, z);
     DF r;
@@ -391,7 +391,7 @@ __device__ __forceinline__ DF row_sum_dfv(const MatView<float> &m, const float *
 
 template <typename Z, int TPR>
 __device__ __forceinline__ double row_sum_df(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             RowPreDf &p, const Z *__restrict__ z)
+                                             RowPreDf &p, const Z *z)
 {
     DF acc = row_sum_df_acc<Z, TPR>(m, lo, row, p, z);
     return (double)acc.hi + (double)acc.lo;

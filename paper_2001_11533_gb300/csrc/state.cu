@@ -280,7 +280,7 @@ __device__ __forceinline__ double scg_head(double r) { return r; }
 
 template <typename M>
 __global__ void __launch_bounds__(SCG_TPB<typename M::Z>, 1)
-    k_state_cg(const __grid_constant__ ScgArgs<typename M::Z> a, const double *__restrict__ f, double *__restrict__ y,
+    k_state_cg(const __grid_constant__ ScgArgs<typename M::Z> a, const double *f, double *__restrict__ y,
                CgScal *scal, double tol2, int maxit)
 {
     typedef typename M::Z T;

@@ -151,17 +151,17 @@ int transfer_setup(amgh_problem *p, Arena &ar, StateLevel &S, const DevCsr &as)
 // b_c = S^T b - (A S)^T x, with the coarse level's first smoother step from
 // zero d_c = x_c = c0 D_c^-1 b_c where that level smooths (d not null)
 template <typename T, int TPR>
-__global__ void k_restrict_pair(MatView<T> W, const T *__restrict__ s, const T *__restrict__ b,
-                                const T *__restrict__ x, T *__restrict__ bc, const T *__restrict__ invd,
-                                T *__restrict__ d, T *__restrict__ xc, T c0, const int *__restrict__ skip)
+__global__ void k_restrict_pair(MatView<T> W, const T *__restrict__ sv, const T *b, const T *x,
+                                T *__restrict__ bc, const T *__restrict__ invd, T *__restrict__ d,
+                                T *__restrict__ xc, T c0, const int *skip)
 {
     int i = my_row<TPR>();
     bool lead = i < W.rows && row_leader<TPR>();
     RowPrePair<T> pre;
     T ir = 0;
-    PDL_ENTER_LOADING(skip, (row_prefetch_pair<T, TPR>(W, s, i, pre)); if (lead && d) ir = invd[i])
+    PDL_ENTER_LOADING(skip, (row_prefetch_pair<T, TPR>(W, sv, i, pre)); if (lead && d) ir = invd[i])
     T v = row_restrict_pair<T, TPR>(
-        W, s, i, pre, [&](int c) { return __ldg(&b[c]); }, [&](int c) { return __ldg(&x[c]); });
+        W, sv, i, pre, [&](int c) { return b[c]; }, [&](int c) { return x[c]; });
     if (lead) {
         bc[i] = v;
         if (d) {
@@ -174,25 +174,25 @@ __global__ void k_restrict_pair(MatView<T> W, const T *__restrict__ s, const T *
 
 // x_n = x + S e + d, d = c D^-1 (b - A x - (A S) e)
 template <typename T, int TPR>
-__global__ void k_prolong_pair(MatView<T> A, MatView<T> W, const T *__restrict__ s, const T *__restrict__ invd,
-                               const T *__restrict__ b, const T *__restrict__ x, const T *__restrict__ e,
-                               T *__restrict__ d, T *__restrict__ xn, T c, const int *__restrict__ skip)
+__global__ void k_prolong_pair(MatView<T> A, MatView<T> W, const T *__restrict__ sv, const T *__restrict__ invd,
+                               const T *b, const T *x, const T *e, T *__restrict__ d, T *__restrict__ xn, T c,
+                               const int *skip)
 {
     int r = my_row<TPR>();
     bool lead = r < A.rows && row_leader<TPR>();
     RowPre<T> pa;
     RowPrePair<T> pw;
     T ir = 0;
-    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pa)); (row_prefetch_pair<T, TPR>(W, s, r, pw));
+    PDL_ENTER_LOADING(skip, (row_prefetch<T, TPR>(A, r, pa)); (row_prefetch_pair<T, TPR>(W, sv, r, pw));
                       if (lead) ir = invd[r])
     T br = 0, xr = 0;
     if (lead) {
         br = b[r];
         xr = x[r];
     }
-    T ax = row_sum_pre<T, TPR>(A, r, pa, [&](int j) { return __ldg(&x[j]); });
+    T ax = row_sum_pre<T, TPR>(A, r, pa, [&](int j) { return x[j]; });
     T ase, se;
-    row_prolong_pair<T, TPR>(W, s, r, pw, [&](int j) { return __ldg(&e[j]); }, ase, se);
+    row_prolong_pair<T, TPR>(W, sv, r, pw, [&](int j) { return e[j]; }, ase, se);
     if (lead) {
         T dn, xv;
         prolong_point(br, ax, ase, se, ir, xr, c, dn, xv);
