@@ -165,13 +165,11 @@ __device__ __forceinline__ typename ScgSum<M, PROD>::V scg_row(const ScgCta<type
             w[j] = PAIR && ok ? lo[(e0 + j) * m.width] : (T)0;
         }
     };
+    const bool idle = sizeof(T) == 8 && t >= m.width; // a warp without entries (the width is a multiple of 32)
     scg_arrive(c.ctas);
-    if (sizeof(T) == 8 && t >= m.width) { // a warp without entries (the width is a multiple of 32)
-        scg_wait(c.ctas);
-        return Sum::zero();
-    }
-    load(0);
-    scg_wait(c.ctas);
+    if (!idle) load(0);
+    scg_wait(c.ctas); // one barrier for all warps
+    if (idle) return Sum::zero();
     typename Sum::V s = Sum::zero();
     for (int e = 0;;) {
 #pragma unroll
