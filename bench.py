@@ -37,7 +37,7 @@ os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 # kernel classes timed together in one instrumented pass (bit c = class c of
 # amgh_kernel_class_stats): each level-0 class alone, then all the others
 TIMING_GROUPS = [1 << 0, 1 << 2, 1 << 4, 1 << 6, 1 << 8, 1 << 10,
-                 ((1 << 15) - 1) & ~((1 << 0) | (1 << 2) | (1 << 4) | (1 << 6) | (1 << 8) | (1 << 10))]
+                 ((1 << 16) - 1) & ~((1 << 0) | (1 << 2) | (1 << 4) | (1 << 6) | (1 << 8) | (1 << 10))]
 METRIC = "Hessian-CG time-to-1e-8 and Hessian matvecs/s, mixed vs FP64, same GB300"
 PRECISION = {"fp64": 0, "refine": 1, "mixed": 2}
 UNIT = "Hessian-matvecs/s"
@@ -487,7 +487,7 @@ def run_cube(args, rank, world, local):
         if form in ("mixed", "mixed_matrix_free"):
             flush.zero_()
             # kernels of 10 us and more here: one pass times every class
-            _, ks, _ = step(precision, timing=(1 << 15) - 1, mf=mf)
+            _, ks, _ = step(precision, timing=(1 << 16) - 1, mf=mf)
             res["roofline"] = roofline_from({"kstats": ks["chebl0"]}, args, kernel_note="level-0 Chebyshev "
                                             "smoother step on the 3D uniform-width SELL-32 matrix (int32 columns)",
                                             traffic=None)

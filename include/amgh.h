@@ -423,7 +423,9 @@ int amgh_reset_counters(amgh_problem *p);
  * graphs, and every solve-phase launch of the single-column path is bracketed
  * by CUDA events on the problem's stream and filed under its kernel class
  * (0 .. AMGH_KCLASSES-1; the launches the device skips, the V-cycle of a CG
- * iteration that converged, are not filed).  amgh_kernel_stats returns class
+ * iteration that converged, are not filed).  A CG solve that runs as one
+ * launch is filed whole, with the bytes of its iterations, under class
+ * "cg_one_launch".  amgh_kernel_stats returns class
  * 0, the level-0 Chebyshev smoother step (SpMV fused with the smoother
  * update); amgh_kernel_class_stats any class, with its name.  Each returns
  * the number of timed launches, their summed duration in ms, and their
@@ -434,7 +436,7 @@ int amgh_reset_counters(amgh_problem *p);
  * amgh_kernel_timing_mask times only the classes whose bit is set in mask
  * (bit c = class c; 0 turns timing off), leaving the others to run as usual.
  * Errors: INVALID_ARG for a class out of range. */
-#define AMGH_KCLASSES 15
+#define AMGH_KCLASSES 16
 int amgh_kernel_timing(amgh_problem *p, int enable);
 int amgh_kernel_timing_mask(amgh_problem *p, unsigned mask);
 int amgh_kernel_stats(amgh_problem *p, int64_t *launches, double *ms, double *bytes);

@@ -60,7 +60,7 @@ class amgh_solve_info(C.Structure):
 
 
 _P, _I, _I64, _D = C.c_void_p, C.c_int, C.c_int64, C.c_double
-KCLASSES = 15  # AMGH_KCLASSES
+KCLASSES = 16  # AMGH_KCLASSES
 _SIGS = {
     "amgh_amg_opts_default": ([_P], None),
     "amgh_solve_opts_default": ([_P], None),

@@ -2387,16 +2387,19 @@ int persistent_mass_single(amgh_problem *p, int l, const double *b, double *x, i
     auto hi = [&](double *v) { return (float *)v; };
     auto lo = [&](double *v) { return (float *)v + n; };
     double tol = p->sopts.mass_tol;
+    timer_begin(p, KC_VEC);
     pdl_launch(kbd_norm<1>, dim3(vblocks(n)), dim3(TPB), 0, p->stream, n, b, bs, tol * tol, maxit, C.red.partials,
                C.red.ticket);
     LAUNCH_CHECK();
     pdl_launch(kbd_start<1>, dim3(vblocks(n)), dim3(TPB), 0, p->stream, (int64_t)n, b, hi(C.mx), lo(C.mx), hi(C.mr),
                lo(C.mr), (float *)C.mz, (const float *)C.mu_invdiag32, (const BScal *)bs);
     LAUNCH_CHECK();
+    timer_end(p, KC_VEC, 32.0 * n); // b twice, x and r
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     MatView<float> A = bview<float>(a);
     cudaError_t err = cudaSuccess;
+    timer_begin(p, KC_CGONE);
     if (!with_tpr(A.tpr, [&](auto t) {
             constexpr int TPR = decltype(t)::value;
             auto kern = kbp_mass_cg<TPR, 1>;
@@ -2431,15 +2434,19 @@ int persistent_mass_single(amgh_problem *p, int l, const double *b, double *x, i
         amgh_note_error((int)err, __FILE__, __LINE__);
         return AMGH_ERR_CUDA;
     }
+    timer_end(p, KC_CGONE, 0.0);
+    const size_t solve = p->timer.pending_bytes.size(); // its bytes follow, once the count is known
+    timer_begin(p, KC_VEC);
     pdl_launch(kbd_out<1>, dim3(vblocks(n)), dim3(TPB), 0, p->stream, (int64_t)n, (const float *)hi(C.mx),
                (const float *)lo(C.mx), (const BScal *)bs, x);
     LAUNCH_CHECK();
+    timer_end(p, KC_VEC, 16.0 * n);
     CgScal h;
     CU(cudaMemcpyAsync(&h, &bs->c[0], sizeof(CgScal), cudaMemcpyDeviceToHost, p->stream));
     TRY(sync_stream(p));
     // algorithmic bytes: per iteration those of the graph-replayed pair (the
     // double-float SpMV with its dots, the update with the Jacobi direction)
-    count_bytes((double)h.iters * (spmv_bytes(a, 4) + 4.0 * a.nnz + 12.0 * n + 84.0 * n) + 48.0 * n);
+    timer_add_bytes(p, KC_CGONE, solve, (double)h.iters * (spmv_bytes(a, 4) + 4.0 * a.nnz + 12.0 * n + 84.0 * n));
     p->c_mass_lvl[l] += h.iters;
     p->c_mass += h.iters;
     if (iters) *iters = h.iters;

@@ -330,6 +330,7 @@ enum KClass {
     KC_COARSE,    // dense coarsest solve, fused coarse V-cycle
     KC_SPMV,      // other sparse products (M_yu, M_y, M_u, P, P^T, ...)
     KC_VEC,       // other vector kernels
+    KC_CGONE,     // a whole CG solve as one launch (state.cu, mass.cu, persistent mass CG)
     KC_N
 };
 static_assert(KC_N == AMGH_KCLASSES, "kernel classes of the ABI");
@@ -655,6 +656,9 @@ int block_solve(amgh_problem *p, const double *yd, int ncols, double *u, const a
 // a solve-phase kernel of class cls; timer_end always counts the bytes
 void timer_begin(amgh_problem *p, int cls);
 void timer_end(amgh_problem *p, int cls, double bytes);
+// bytes known only later (a CG that counts its iterations) of the timing that
+// was number `timing`: pending_bytes.size() after its timer_end
+void timer_add_bytes(amgh_problem *p, int cls, size_t timing, double bytes);
 int timer_collect(amgh_problem *p);
 // drop the pending timings recorded since `mark` (launches that the device
 // skipped: the V-cycle of a CG iteration that converged)

@@ -523,13 +523,18 @@ int state_solve(amgh_problem *p, int l, const double *f, double *y, double tol, 
     int maxit = p->sopts.inner_max_iter;
     int prec = p->aopts.precision;
     bool one_launch = false;
+    const size_t mark = p->timer.ev.size();
+    timer_begin(p, KC_CGONE);
     TRY(state_cluster(p, l, f, y, tol, maxit, &one_launch));
-    if (one_launch) {
+    if (!one_launch) timer_drop_from(p, mark);
+    else {
+        timer_end(p, KC_CGONE, 0.0);
         CgScal h;
         TRY(read_scal(p, S.scal, &h));
         // per iteration as the graph-replayed one: V-cycle, product with its dots, update
         const double mat = prec == 2 ? spmv_bytes(S.A, 4) + 4.0 * S.A.nnz : spmv_bytes(S.A, 8);
-        count_bytes(h.iters * (vcycle_bytes(p, l, prec == 2 ? 4 : 8) + mat + 88.0 * n));
+        timer_add_bytes(p, KC_CGONE, p->timer.pending_bytes.size(),
+                        h.iters * (vcycle_bytes(p, l, prec == 2 ? 4 : 8) + mat + 88.0 * n));
         p->c_inner_lvl[l] += h.iters;
         p->c_inner += h.iters;
         if (iters) *iters = h.iters;
@@ -576,21 +581,22 @@ int mass_solve(amgh_problem *p, int l, const double *b, double *x, int64_t *iter
     bool df = p->aopts.precision == 2;
     bool one_launch = false;
     const size_t mark = p->timer.ev.size();
-    timer_begin(p, KC_VEC);
+    timer_begin(p, KC_CGONE);
     TRY(mass_cluster(p, C, df, b, x, C.mscal, 1, p->sopts.mass_tol, p->sopts.mass_max_iter, &one_launch));
-    if (one_launch) {
-        timer_end(p, KC_VEC, 48.0 * n);
+    if (!one_launch) timer_drop_from(p, mark);
+    else {
+        timer_end(p, KC_CGONE, 0.0);
         CgScal h;
         TRY(read_scal(p, C.mscal, &h));
         // per iteration as the graph-replayed pair: the product with its dots, the update
         const double mat = df ? spmv_bytes(C.Mu, 4) + 4.0 * C.Mu.nnz : spmv_bytes(C.Mu, 8);
-        count_bytes(h.iters * (mat + (df ? 96.0 : 112.0) * n));
+        timer_add_bytes(p, KC_CGONE, p->timer.pending_bytes.size(),
+                        h.iters * (mat + (df ? 96.0 : 112.0) * n) + 48.0 * n);
         p->c_mass_lvl[l] += h.iters;
         p->c_mass += h.iters;
         if (iters) *iters = h.iters;
         return cg_status(h);
     }
-    timer_drop_from(p, mark);
     if (df && p->aopts.persistent_cg && !p->parent && !p->in_batch && !p->capturing)
         return persistent_mass_single(p, l, b, x, iters);
     if (df) {

@@ -295,7 +295,7 @@ const char *kclass_name(int c)
     static const char *names[KC_N] = {"cheb_step_l0", "cheb_step_coarse", "residual_l0", "residual_coarse",
                                       "restrict_l0", "restrict_coarse", "prolong_l0", "prolong_coarse",
                                       "cg_spmv_l0", "cg_spmv_coarse", "cg_update_l0", "cg_update_coarse",
-                                      "coarsest", "spmv_other", "vector_other"};
+                                      "coarsest", "spmv_other", "vector_other", "cg_one_launch"};
     return c >= 0 && c < KC_N ? names[c] : "?";
 }
 
@@ -316,6 +316,14 @@ void timer_end(amgh_problem *p, int cls, double bytes)
     p->timer.ev.push_back(b);
     p->timer.cls.push_back(cls);
     p->timer.pending_bytes.push_back(bytes);
+}
+
+void timer_add_bytes(amgh_problem *p, int cls, size_t timing, double bytes)
+{
+    count_bytes(bytes);
+    if (!p->timer.enabled || !(p->timer.mask >> cls & 1u) || timing < 1 || timing > p->timer.pending_bytes.size())
+        return;
+    p->timer.pending_bytes[timing - 1] += bytes;
 }
 
 void timer_drop_from(amgh_problem *p, size_t mark)
