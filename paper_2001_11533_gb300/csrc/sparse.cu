@@ -130,7 +130,8 @@ int csr_to_sell(Arena &ar, DevCsr &a, int /*want32*/, cudaStream_t s)
         int hb = 0;
         CU(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));
-        if (!hb) a.sl_ci16 = d16;
+        if (hb) ar.release(d16);
+        else a.sl_ci16 = d16;
     }
     CU(cudaStreamSynchronize(s));
     return AMGH_OK;
@@ -371,6 +372,9 @@ int prepare_operator(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
             TRY(prepare_layout(ar, c, s, force_tpr));
             if (c.tpr <= 1) { // SELL-32 has its own copies
                 for (void *q : {(void *)c.rp, (void *)c.ci, (void *)c.v}) ar.release(q);
+            } else if (c.x16) { // its columns are read as int16 offsets
+                ar.release(c.ci);
+                c.xi = nullptr;
             }
             // everything but the canonical CSR
             c.rp = a.rp;
@@ -428,7 +432,8 @@ int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
         }
     }
     CU(cudaStreamSynchronize(s));
-    if (d16 && !hb) a.x16 = d16;
+    if (hb) ar.release(d16);
+    else a.x16 = d16;
     return AMGH_OK;
 }
 
