@@ -54,6 +54,9 @@ def parse():
                          "cube, 10 slabs of kappa in {1, 1e6}, beta 1e-6")
     ap.add_argument("--N", type=int, default=None, help="grid size (default 1025 for lshape, 257 for cube)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--detail", default=os.path.join(ROOT, "bench_detail.json"),
+                    help="file that receives the full record (kernel classes, forms, batch, cube); the printed "
+                         "line holds the headline keys")
     ap.add_argument("--coarse-max", type=int, default=1000,
                     help="AMG stops at or below this many rows (1000: 4 levels, 784k..847 on the L-shape)")
     ap.add_argument("--degree", type=int, default=2, help="Chebyshev smoother degree")
@@ -696,6 +699,37 @@ def run_reference(args, rank, world):
     print(json.dumps(line), flush=True)
 
 
+def headline(line, detail):
+    """The keys of the full record that the printed line keeps: what a reader of
+    the last lines of the output needs, in under 2,500 characters; the full
+    record is in the file `detail`."""
+    def take(d, *keys):
+        return {k: (round(v, 4) if isinstance(v, float) else v) for k, v in d.items() if k in keys}
+
+    out = {k: v for k, v in line.items() if not isinstance(v, dict) or k == "config"}
+    out["clocks"] = take(line["clocks"], "sm_mhz", "sm_max_mhz", "reasons")
+    if line.get("roofline"):
+        out["roofline"] = take(line["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic",
+                               "peak_source", "launches", "avg_us")
+    if line.get("solve_phase"):
+        out["solve_phase"] = take(line["solve_phase"], "solve_s", "achieved_GBs", "frac")
+    if line.get("e2e"):
+        out["e2e"] = {k: line["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step",
+                                                  "ms_per_step") if k in line["e2e"]}
+    out["forms"] = {f: take(r, "value", "ms_per_step", "outer_iters", "setup_s") for f, r in line["forms"].items()}
+    for part in ("batch", "cube"):
+        if part in line:
+            out[part] = {f: round(r["hessian_matvecs_per_s"], 4) for f, r in line[part].items()
+                         if isinstance(r, dict) and "hessian_matvecs_per_s" in r}
+            out[part]["unit"] = UNIT
+    if "dense_fp64" in line:
+        out["dense_fp64"] = take(line["dense_fp64"]["spd_inverse"], "n", "ms", "tflops", "status")
+    if "cpu_baseline" in line:
+        out["cpu_baseline"] = take(line["cpu_baseline"], "value", "unit", "cores", "kind")
+    out["detail"] = detail
+    return out
+
+
 # ------------------------------------------------------------------------- main
 def single_step(args):
     """One step of the first form, untimed, for profilers (ncu launch lists)."""
@@ -848,7 +882,12 @@ def main():
         line["dense_fp64"] = dense_fp64(head["levels"]["state"][-1])
     if world == 1 and not args.no_cpu_baseline and args.workload == "lshape":
         line["cpu_baseline"] = cpu_baseline(w, args)
-    print(json.dumps(line), flush=True)
+    try:
+        with open(args.detail, "w") as f:
+            json.dump(line, f, indent=1)
+    except OSError as e:  # the record is a by-product: the line below counts
+        print(f"bench: {args.detail} not written ({e})", file=sys.stderr)
+    print(json.dumps(headline(line, os.path.basename(args.detail))), flush=True)
 
 
 if __name__ == "__main__":
