@@ -43,8 +43,13 @@
 // by butterflies over nearly empty lanes, one addition of a whole warp a step;
 // with 256, at least two entries a lane and idle warps skipping the phase 2,025
 // rows take 452 us instead of 665 (33^2 cost and gradient 1.40 -> 1.12 ms).  FP32
-// solves alone gain 7 % by the same, but whole calls lose 1 % (65^2 solve 13.43 ->
-// 13.55 ms, 201^2 preconditioner 4.51 -> 4.56), so they keep the wider form.
+// additions are cheap, so its lanes pay: 512 threads -> 256 and two entries a lane
+// are 243 -> 230 us on short rows (33^2) but 84 -> 94 on a level of 115 rows of up
+// to 24 entries, and a lane's 16 entries then end at rows half as long, so that
+// hierarchies fall back to the replayed kernels: 47^2 over four levels 444 -> 683
+// us, a cube's level of 449 rows of up to 78 entries 318 -> 428.  Whole calls on
+// short rows cannot tell them apart (65^2 solve 13.59 and 13.64 ms, 201^2
+// preconditioner 4.48 and 4.49).
 template <typename T>
 constexpr int SCG_TPB = sizeof(T) == 8 ? 256 : 512;
 #define SCG_ROWS 128 // rows of the solved level per CTA
