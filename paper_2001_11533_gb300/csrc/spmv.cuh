@@ -336,11 +336,11 @@ __device__ __forceinline__ void row_prefetch_df(const MatView<float> &m, const f
     }
 }
 
-// sum_j a_rj xf(j) in double-float from a prefetched row, not normalised;
+// sum_j a_rj z_j in double-float from a prefetched row, not normalised;
 // every lane of the group returns it
-template <typename Z, int TPR, typename F>
-__device__ __forceinline__ DF row_sum_df_xf(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                            RowPreDf &p, F xf)
+template <typename Z, int TPR>
+__device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const float *__restrict__ lo, int row,
+                                            RowPreDf &p, const Z *z)
 {
     constexpr int STEP = TPR == 1 ? 32 : TPR;
     DF acc = {0.f, 0.f};
@@ -349,7 +349,7 @@ __device__ __forceinline__ DF row_sum_df_xf(const MatView<float> &m, const float
         auto chunk = [&](int k0) {
             Z zv[ROW_UNROLL];
 #pragma unroll
-            for (int j = 0; j < ROW_UNROLL; j++) zv[j] = k0 + STEP * j < end ? xf(p.h.cc[j]) : (Z)0;
+            for (int j = 0; j < ROW_UNROLL; j++) zv[j] = k0 + STEP * j < end ? z[p.h.cc[j]] : (Z)0;
 #pragma unroll
             for (int j = 0; j < ROW_UNROLL; j++)
                 if (k0 + STEP * j < end) df_term<Z>(acc, p.h.vv[j], p.vl[j], zv[j]);
@@ -369,13 +369,6 @@ __device__ __forceinline__ DF row_sum_df_xf(const MatView<float> &m, const float
         }
     }
     return acc;
-}
-
-template <typename Z, int TPR>
-__device__ __forceinline__ DF row_sum_df_acc(const MatView<float> &m, const float *__restrict__ lo, int row,
-                                             RowPreDf &p, const Z *z)
-{
-    return row_sum_df_xf<Z, TPR>(m, lo, row, p, [&](int c) { return z[c]; });
 }
 
 // sum_j a_rj z_j in double-float (normalised)
