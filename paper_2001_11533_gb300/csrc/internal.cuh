@@ -459,8 +459,8 @@ void mis_set_round_cap(int cap);
 void prol_set_row_cap(int cap);
 // b = (float)a
 int to_f32(amgh_problem *p, const double *a, int64_t n, float *b);
-// the layout itself, without leaving out exact zeros
-int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr);
+// the layout itself, without leaving out exact zeros (longest: the longest row, -1: not known)
+int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr, int longest = -1);
 // build a.lo32 (after prepare_operator)
 int build_lo_parts(Arena &ar, DevCsr &a, cudaStream_t s);
 int csr_transpose(Arena &ar, const DevCsr &a, DevCsr &t, cudaStream_t s);

@@ -133,7 +133,6 @@ int csr_to_sell(Arena &ar, DevCsr &a, int /*want32*/, cudaStream_t s)
         if (hb) ar.release(d16);
         else a.sl_ci16 = d16;
     }
-    CU(cudaStreamSynchronize(s));
     return AMGH_OK;
 }
 
@@ -302,13 +301,26 @@ static int max_row_length(const DevCsr &a, cudaStream_t s, int *out)
     return AMGH_OK;
 }
 
-__global__ void k_count_nonzero(int rows, const int *__restrict__ rp, const double *__restrict__ v, int *__restrict__ cnt)
+// non-zero entries of every row; longest[0], longest[1]: most entries of a row,
+// with and without the exact zeros
+__global__ void k_count_nonzero(int rows, const int *__restrict__ rp, const double *__restrict__ v, int *__restrict__ cnt,
+                                int *__restrict__ longest)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    int c = 0;
-    for (int k = rp[i]; k < rp[i + 1]; k++) c += v[k] != 0.0;
-    cnt[i] = c;
+    int c = 0, len = 0;
+    if (i < rows) {
+        len = rp[i + 1] - rp[i];
+        for (int k = rp[i]; k < rp[i + 1]; k++) c += v[k] != 0.0;
+        cnt[i] = c;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
+        c = max(c, __shfl_xor_sync(0xffffffffu, c, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&longest[0], len);
+        atomicMax(&longest[1], c);
+    }
 }
 
 __global__ void k_drop_zeros(int rows, const int *__restrict__ rp, const int *__restrict__ ci,
@@ -353,48 +365,50 @@ int prepare_operator(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
 {
     if (a.rows > 0 && a.nnz > 0 && force_tpr <= 1) {
         Scratch sc;
-        int *cnt = nullptr, *rp2 = nullptr;
+        int *cnt = nullptr, *rp2 = nullptr; // rp2: row pointers, then the two longest rows: one read
         TRY(sc.alloc(&cnt, a.rows + 1));
-        TRY(sc.alloc(&rp2, a.rows + 1));
-        k_count_nonzero<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.v, cnt);
+        TRY(sc.alloc(&rp2, a.rows + 3));
+        CU(cudaMemsetAsync(rp2 + a.rows + 1, 0, 2 * sizeof(int), s));
+        k_count_nonzero<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.v, cnt, rp2 + a.rows + 1);
         LAUNCH_CHECK();
-        int nz = 0;
-        TRY(exclusive_scan<int>(cnt, rp2, a.rows, s, &nz));
-        if ((double)nz < 0.95 * a.nnz) {
-            DevCsr c = a;
-            c.nnz = nz;
-            TRY(ar.alloc(&c.rp, a.rows + 1));
-            TRY(ar.alloc(&c.ci, nz));
-            TRY(ar.alloc(&c.v, nz));
-            CU(cudaMemcpyAsync(c.rp, rp2, sizeof(int) * (a.rows + 1), cudaMemcpyDeviceToDevice, s));
-            k_drop_zeros<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.ci, a.v, rp2, c.ci, c.v);
-            LAUNCH_CHECK();
-            TRY(prepare_layout(ar, c, s, force_tpr));
-            if (c.tpr <= 1) { // SELL-32 has its own copies
-                for (void *q : {(void *)c.rp, (void *)c.ci, (void *)c.v}) ar.release(q);
-            } else if (c.x16) { // its columns are read as int16 offsets
-                ar.release(c.ci);
-                c.xi = nullptr;
-            }
-            // everything but the canonical CSR
-            c.rp = a.rp;
-            c.ci = a.ci;
-            c.v = a.v;
-            c.nnz = a.nnz;
-            TRY(max_row_length(a, s, &c.longest));
-            c.nnz_solve = nz;
-            a = c;
-            return AMGH_OK;
+        TRY(exclusive_scan<int>(cnt, rp2, a.rows, s, nullptr));
+        int found[3] = {0, 0, 0};
+        CU(cudaMemcpyAsync(found, rp2 + a.rows, sizeof(found), cudaMemcpyDeviceToHost, s));
+        CU(cudaStreamSynchronize(s));
+        const int nz = found[0];
+        if ((double)nz >= 0.95 * a.nnz) return prepare_layout(ar, a, s, force_tpr, found[1]);
+        DevCsr c = a;
+        c.nnz = nz;
+        TRY(ar.alloc(&c.rp, a.rows + 1));
+        TRY(ar.alloc(&c.ci, nz));
+        TRY(ar.alloc(&c.v, nz));
+        CU(cudaMemcpyAsync(c.rp, rp2, sizeof(int) * (a.rows + 1), cudaMemcpyDeviceToDevice, s));
+        k_drop_zeros<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.ci, a.v, rp2, c.ci, c.v);
+        LAUNCH_CHECK();
+        TRY(prepare_layout(ar, c, s, force_tpr, found[2]));
+        if (c.tpr <= 1) { // SELL-32 has its own copies
+            for (void *q : {(void *)c.rp, (void *)c.ci, (void *)c.v}) ar.release(q);
+        } else if (c.x16) { // its columns are read as int16 offsets
+            ar.release(c.ci);
+            c.xi = nullptr;
         }
+        // everything but the canonical CSR
+        c.rp = a.rp;
+        c.ci = a.ci;
+        c.v = a.v;
+        c.nnz = a.nnz;
+        c.longest = found[1];
+        c.nnz_solve = nz;
+        a = c;
+        return AMGH_OK;
     }
     return prepare_layout(ar, a, s, force_tpr);
 }
 
-int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
+int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr, int longest)
 {
     double avg = a.rows > 0 ? (double)a.nnz / a.rows : 0.0;
-    int longest = 0;
-    TRY(max_row_length(a, s, &longest));
+    if (longest < 0) TRY(max_row_length(a, s, &longest));
     a.longest = longest;
     // SELL-32 for short rows, and for rows up to 16 long when every row has
     // nearly the longest length (uniform-width SELL: the staged smoother);
@@ -429,9 +443,9 @@ int prepare_layout(Arena &ar, DevCsr &a, cudaStream_t s, int force_tpr)
             k_csr_delta<<<ceil_div(a.rows, 256), 256, 0, s>>>(a.rows, a.rp, a.ci, d16, bad);
             LAUNCH_CHECK();
             CU(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+            CU(cudaStreamSynchronize(s));
         }
     }
-    CU(cudaStreamSynchronize(s));
     if (hb) ar.release(d16);
     else a.x16 = d16;
     return AMGH_OK;

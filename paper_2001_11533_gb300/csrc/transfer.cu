@@ -142,7 +142,6 @@ int transfer_setup(amgh_problem *p, Arena &ar, StateLevel &S, const DevCsr &as)
     LAUNCH_CHECK();
     TRY(pair_layout(p, ar, S.up, s, S.A.tpr < 1 ? 1 : S.A.tpr));
     TRY(pair_layout(p, ar, S.down, t, 0));
-    CU(cudaStreamSynchronize(st)); // the scratch arrays
     S.paired = true;
     return AMGH_OK;
 }
