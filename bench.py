@@ -551,7 +551,9 @@ def kernel_table(classes):
     """Per kernel class from the instrumented passes: launches, mean duration, achieved
     GB/s on algorithmic bytes, fraction of the measured HBM copy peak, and share of
     the timed kernel time.  A coarse class moving under 32 MB per launch works on
-    operands that stay in the 129 MB L2: its bytes/s is labelled L2-resident."""
+    operands that stay in the 129 MB L2: its bytes/s is labelled L2-resident.  A CG
+    solve in one launch counts the bytes of all its iterations, which it reads
+    from shared memory, registers or L2."""
     peak, _ = hbm_peak()
     total = sum(c["ms"] for c in classes.values()) or 1.0
     out = {}
@@ -563,7 +565,8 @@ def kernel_table(classes):
         out[name] = {"launches": c["launches"], "avg_us": round(1000.0 * c["ms"] / c["launches"], 2),
                      "share": round(c["ms"] / total, 4), "achieved_GBs": round(gbs, 1),
                      "frac_of_hbm": round(gbs / peak, 4), "mb_per_launch": round(per / 1e6, 2),
-                     "residency": "hbm" if (name.endswith("_l0") or per >= 32e6) else "l2-resident"}
+                     "residency": "cached (all iterations)" if name == "cg_one_launch" else
+                     "hbm" if (name.endswith("_l0") or per >= 32e6) else "l2-resident"}
     return out
 
 

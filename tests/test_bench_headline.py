@@ -54,6 +54,12 @@ def test_line_is_short_and_complete():
     assert line["forms"]["mixed"]["ms_per_step"] == 116.1974 and line["detail"] == "bench_detail.json"
 
 
+def test_whole_solves_are_not_labelled_as_hbm_traffic():
+    t = bench.kernel_table({"cg_one_launch": {"launches": 2, "ms": 0.4, "bytes": 4.8e8},
+                            "cg_spmv_l0": {"launches": 2, "ms": 0.04, "bytes": 1.4e8}})
+    assert t["cg_one_launch"]["residency"].startswith("cached") and t["cg_spmv_l0"]["residency"] == "hbm"
+
+
 def test_parts_that_were_not_run_are_left_out():
     full = record()
     full["batch"]["mixed"] = {"status": -5}  # a part that failed has no rate
