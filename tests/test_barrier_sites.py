@@ -1,6 +1,6 @@
-"""All warps of a CTA meet a barrier at the same place in the source: CUDA promises
-nothing for a __syncthreads() that some warps reach on another path.  (Read from
-the sources; no GPU needed.)"""
+"""Warps that wait at different places of the source do so by PTX barriers, which
+count the warps that arrive wherever they do; CUDA defines __syncthreads() only
+where all of them reach the same one.  (Read from the sources; no GPU needed.)"""
 import os
 import re
 
@@ -12,8 +12,9 @@ def body(src, name):
     return re.sub(r"//.*", "", m.group(1))
 
 
-def test_rows_of_the_cluster_state_solve_wait_at_one_place():
-    b = body(open(os.path.join(CSRC, "state.cu")).read(), "scg_row")
-    assert b.count("scg_arrive(") == 1 and b.count("scg_wait(") == 1
-    assert "return" not in b[:b.index("scg_wait(")].split("auto load")[0]
-    assert "return" not in b[b.index("scg_arrive("):b.index("scg_wait(")]
+def test_waits_of_the_cluster_state_solve_are_ptx_barriers():
+    src = open(os.path.join(CSRC, "state.cu")).read()
+    row, wait = body(src, "scg_row"), body(src, "scg_wait")
+    assert row.count("scg_arrive(") == 1 and row.count("scg_wait(") == 2  # with and without entries
+    assert "__syncthreads" not in row and "__syncthreads" not in wait
+    assert "barrier.cta.sync.aligned 0;" in wait and "barrier.cluster.wait" in wait
